@@ -57,6 +57,35 @@ struct CtaColl : std::false_type {};
 template <class Pb>
 struct CtaColl<Pb, std::void_t<decltype(Pb::kCta)>> : std::integral_constant<bool, Pb::kCta> {};
 
+// Lanes per trajectory (1; the neural Robertson's lane-group form: 16). The
+// lanes of a group carry the same trajectory; its first lane takes the tickets,
+// reserves arena slots and writes the results.
+template <class Pb, class = void>
+struct GroupOf : std::integral_constant<int, 1> {};
+template <class Pb>
+struct GroupOf<Pb, std::void_t<decltype(Pb::kGroup)>> : std::integral_constant<int, Pb::kGroup> {};
+// The per-lane form of a problem (the passes that give each trajectory one lane).
+template <class Pb, class = void>
+struct LaneOf {
+  using type = Pb;
+};
+template <class Pb>
+struct LaneOf<Pb, std::void_t<typename Pb::Lane>> {
+  using type = typename Pb::Lane;
+};
+template <class Pb>
+__device__ __forceinline__ bool group_leader() {
+  return (threadIdx.x & (GroupOf<Pb>::value - 1)) == 0;
+}
+// The leader's value on every lane of its group (the whole warp calls it).
+template <class Pb>
+__device__ __forceinline__ long long from_leader(long long v) {
+  if constexpr (GroupOf<Pb>::value == 1)
+    return v;
+  else
+    return __shfl_sync(FULL_MASK, v, 0, GroupOf<Pb>::value);
+}
+
 constexpr int TPB_FWD = 128;
 constexpr int TPB_REV = 128;
 
@@ -295,7 +324,8 @@ struct Rodas5PMethod {  // FP64 only: the stiff W-matrix LU and its solves stay 
                                                  const Carry<Pb, R>&, R (&ynew)[Pb::D], R (&e)[Pb::D],
                                                  Carry<Pb, R>&, StageData<Pb, R>& sd) {
     constexpr int D = Pb::D;
-    const bool ok = rodas_step<Pb>(y, p, h, sd.Y, sd.U, sd.LU, sd.piv, sd.rinv, ynew);
+    typename TapeOf<Pb>::type tape;
+    const bool ok = rodas_step<Pb>(y, p, h, sd.Y, sd.U, sd.LU, sd.piv, sd.rinv, ynew, tape);
 #pragma unroll
     for (int c = 0; c < D; ++c) e[c] = sd.U[7][c];
     return ok;
@@ -346,7 +376,8 @@ struct Rodas5PMethod {  // FP64 only: the stiff W-matrix LU and its solves stay 
     const bool side = (mode == U_SIDE);
     double cv[D], v[D];
     unit_cotangent<Pb, R, USER_COT>(a, k, active, side, us, sd.ynew, lam, cv, loss);
-    rodas_reverse<Pb>(x, p, h, sd.Y, sd.U, sd.LU, sd.piv, sd.rinv, cv, v, pacc);
+    typename TapeOf<Pb>::type tape;
+    rodas_reverse<Pb>(x, p, h, sd.Y, sd.U, sd.LU, sd.piv, sd.rinv, cv, v, pacc, tape);
 #pragma unroll
     for (int c = 0; c < D; ++c) lam[c] = !active ? lam[c] : (side ? add_(lam[c], v[c]) : v[c]);
     return true;
@@ -368,7 +399,8 @@ struct Rodas5PMethod {  // FP64 only: the stiff W-matrix LU and its solves stay 
     constexpr int D = Pb::D;
     double Y[8][D], U[8][D], LU[D][D], rinv[D];
     int piv[D];
-    const bool ok = rodas_step<Pb>(y, p, h, Y, U, LU, piv, rinv, ynew);
+    typename TapeOf<Pb>::type tape;
+    const bool ok = rodas_step<Pb>(y, p, h, Y, U, LU, piv, rinv, ynew, tape);
 #pragma unroll
     for (int c = 0; c < D; ++c) e[c] = U[7][c];
     return ok;
@@ -379,7 +411,8 @@ struct Rodas5PMethod {  // FP64 only: the stiff W-matrix LU and its solves stay 
     constexpr int D = Pb::D;
     double Y[8][D], U[8][D], LU[D][D], rinv[D];
     int piv[D];
-    return rodas_step<Pb>(y, p, h, Y, U, LU, piv, rinv, ys);
+    typename TapeOf<Pb>::type tape;
+    return rodas_step<Pb>(y, p, h, Y, U, LU, piv, rinv, ys, tape);
   }
   template <class Pb, class R>
   __device__ __forceinline__ static bool replay_step(const R (&y)[Pb::D], const R (&p)[Pb::NP], double h,
@@ -387,7 +420,8 @@ struct Rodas5PMethod {  // FP64 only: the stiff W-matrix LU and its solves stay 
     constexpr int D = Pb::D;
     double Y[8][D], U[8][D], LU[D][D], rinv[D];
     int piv[D];
-    return rodas_step<Pb>(y, p, h, Y, U, LU, piv, rinv, ynew);
+    typename TapeOf<Pb>::type tape;
+    return rodas_step<Pb>(y, p, h, Y, U, LU, piv, rinv, ynew, tape);
   }
   template <class Pb, class R, bool USER_COT, class Acc>
   __device__ __forceinline__ static bool unit(const RevArgs& a, long long k, int mode, bool active, int us,
@@ -397,12 +431,13 @@ struct Rodas5PMethod {  // FP64 only: the stiff W-matrix LU and its solves stay 
     constexpr int D = Pb::D;
     double Y[8][D], U[8][D], LU[D][D], rinv[D];
     int piv[D];
-    const bool ok = rodas_step<Pb>(x, p, h, Y, U, LU, piv, rinv, ynew);
+    typename TapeOf<Pb>::type tape;
+    const bool ok = rodas_step<Pb>(x, p, h, Y, U, LU, piv, rinv, ynew, tape);
     if (mode == U_RECOMP) return ok;
     const bool side = (mode == U_SIDE);
     double cv[D], v[D];
     unit_cotangent<Pb, R, USER_COT>(a, k, active, side, us, ynew, lam, cv, loss);
-    rodas_reverse<Pb>(x, p, h, Y, U, LU, piv, rinv, cv, v, pacc);
+    rodas_reverse<Pb>(x, p, h, Y, U, LU, piv, rinv, cv, v, pacc, tape);
 #pragma unroll
     for (int c = 0; c < D; ++c) lam[c] = !active ? lam[c] : (side ? add_(lam[c], v[c]) : v[c]);
     return ok;
@@ -789,7 +824,7 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
     // ---- refill: lanes without a trajectory take the next ticket
     const bool need = (k < 0) && !drained;
     if (__any_sync(FULL_MASK, need)) {
-      const long long got = warp_ticket(a.work, need);
+      const long long got = from_leader<Pb>(warp_ticket(a.work, need && group_leader<Pb>()));
       if (need) {
         if (got < n) {
           k = got;
@@ -1027,7 +1062,7 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
       // arena slots are reserved per warp in blocks (one atomic per block, not
       // per flush); the unused tail of a warp's last block stays empty, since
       // segments are linked, not indexed
-      const unsigned fm = __ballot_sync(FULL_MASK, flush);
+      const unsigned fm = __ballot_sync(FULL_MASK, flush && group_leader<Pb>());
       const int cnt = __popc(fm), rem = (int)(res_end - res_next);
       const int blk = a.arena_block >= 32 ? a.arena_block : ARENA_BLOCK_HOST;
       long long nb = 0;
@@ -1037,7 +1072,7 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
         nb = (long long)__shfl_sync(FULL_MASK, base, 0);
       }
       const int rank = __popc(fm & ((1u << lane_id()) - 1u));
-      const long long idx = rank < rem ? res_next + rank : nb + (rank - rem);
+      const long long idx = from_leader<Pb>(rank < rem ? res_next + rank : nb + (rank - rem));
       if (cnt > rem) {
         res_next = nb + (cnt - rem);
         res_end = nb + blk;
@@ -1046,7 +1081,8 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
       }
       if (flush) {
         stg[0] = __longlong_as_double(prev);
-        if (idx < a.arena_cap) {
+        if (!group_leader<Pb>()) {
+        } else if (idx < a.arena_cap) {
           double2* dst = reinterpret_cast<double2*>(a.arena + idx * a.segw);
           for (int w = 0; w < (a.segw >> 1); ++w) dst[w] = make_double2(stg[(2 * w) * TB], stg[(2 * w + 1) * TB]);
         } else {
@@ -1061,17 +1097,19 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
     }
 
     if (done) {
-      if (a.head) a.head[k] = prev;
-      if (a.S) a.S[k] = S;
-      if (a.natt) a.natt[k] = natt;
-      a.status[k] = status;
+      if (group_leader<Pb>()) {
+        if (a.head) a.head[k] = prev;
+        if (a.S) a.S[k] = S;
+        if (a.natt) a.natt[k] = natt;
+        a.status[k] = status;
 #pragma unroll
-      for (int c = 0; c < D; ++c) a.y_final[c * n + k] = (double)y[c];
-      if (a.step_counts) {
-        a.step_counts[k] = S;
-        a.step_counts[n + k] = natt;
+        for (int c = 0; c < D; ++c) a.y_final[c * n + k] = (double)y[c];
+        if (a.step_counts) {
+          a.step_counts[k] = S;
+          a.step_counts[n + k] = natt;
+        }
+        if (status != TRAJ_OK) *a.any_failed = 1;
       }
-      if (status != TRAJ_OK) *a.any_failed = 1;
       k = -1;
     }
   }
@@ -1229,6 +1267,10 @@ struct WeightAcc<LvUdeCta> {
 template <>
 struct WeightAcc<NeuralRobertson> {
   using type = NrAcc;
+};
+template <>
+struct WeightAcc<NeuralRobertsonGroup> {
+  using type = NrGroupAcc;
 };
 template <class Pb, class R>
 using AccFor = typename std::conditional<HasWeights<Pb>::value, typename WeightAcc<Pb>::type, AccOf<R, Pb::NP>>::type;
@@ -1441,29 +1483,31 @@ __global__ void __launch_bounds__(256) t1_save_kernel(const RevArgs a) {
 template <class M, class Pb, class R, bool USER_COT, bool STAGES = false>
 __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
   constexpr int D = Pb::D, NP = Pb::NP;
-  constexpr bool COLL = HasWeights<Pb>::value;
+  constexpr int G = GroupOf<Pb>::value;
+  constexpr bool STATIC = HasWeights<Pb>::value;  // static schedule, shared weights and their gradient
+  constexpr bool COLL = STATIC && G == 1;          // units run by every lane of the warp together
   constexpr bool CTA = CtaColl<Pb>::value;  // units in lockstep across the CTA, not only the warp
   using Acc = AccFor<Pb, R>;
   extern __shared__ double smem[];
   const int ns = a.n_save;
   double* s_save = smem;
   for (int i = threadIdx.x; i < ns; i += blockDim.x) s_save[i] = a.save_t[i];
-  if constexpr (COLL) Pb::block_setup(a.shared_w);
+  if constexpr (STATIC) Pb::block_setup(a.shared_w);
   __syncthreads();
 
   const long long n = a.n;
   long long k = -1;
   bool drained = false;
   R p[NP], lam[D], yx[D];  // yx: the mesh state the next unit starts from
-  // static schedule (shared-weight problems): lane i takes trajectories i, i + L, i + 2L, ...
-  long long stat_next = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long stat_stride = (long long)gridDim.x * blockDim.x;
+  // static schedule (shared-weight problems): lane (or group) i takes trajectories i, i + L, i + 2L, ...
+  long long stat_next = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / G;
+  const long long stat_stride = (long long)gridDim.x * blockDim.x / G;
 #pragma unroll
   for (int q = 0; q < NP; ++q) p[q] = R(0);
 #pragma unroll
   for (int c = 0; c < D; ++c) lam[c] = yx[c] = R(0);
   Acc pacc;
-  if constexpr (COLL) pacc.init(smem + ((ns + 1) & ~1));
+  if constexpr (STATIC) pacc.init(smem + ((ns + 1) & ~1));
   double loss = 0.0, tx = 0.0;
   long long seg = -1;
   int js = -1, segs_left = 0;
@@ -1472,7 +1516,7 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
     const bool need = (k < 0) && !drained;
     if (__any_sync(FULL_MASK, need)) {
       long long got;
-      if constexpr (COLL) {
+      if constexpr (STATIC) {
         got = need ? stat_next : -1;
         if (need) stat_next += stat_stride;
       } else {
@@ -1483,7 +1527,7 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
           k = got;
           const long long hd = a.head[k];
           if (a.status[k] != TRAJ_OK || hd < 0) {
-            write_nan<NP, D>(a, k);
+            if (group_leader<Pb>()) write_nan<NP, D>(a, k);
             k = -1;
           } else {
 #pragma unroll
@@ -1607,15 +1651,15 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
         mode = U_FAIL;
     }
     if (mode == U_FAIL) {
-      write_nan<NP, D>(a, k);
+      if (group_leader<Pb>()) write_nan<NP, D>(a, k);
       k = -1;
     }
     if (mode == U_DONE) {
-      write_grad<NP, D, R>(a, k, pacc, lam, loss);
+      if (group_leader<Pb>()) write_grad<NP, D, R>(a, k, pacc, lam, loss);
       k = -1;
     }
   }
-  if constexpr (COLL) {
+  if constexpr (STATIC) {
     if (a.wpart) pacc.finish(a.wpart, (size_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
   }
   if constexpr (CTA) Pb::block_teardown(a.tc_error);
@@ -1740,7 +1784,7 @@ inline int sm_count() {
 // ensemble needs).
 template <class Kern>
 inline cudaError_t persistent_launch(Kern kern, int tpb, size_t smem, long long n, cudaStream_t s,
-                                     const void* args_ptr) {
+                                     const void* args_ptr) {  // n: lanes with work
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   int bps = 0;
@@ -1793,36 +1837,37 @@ inline cudaError_t fwd_dispatch(const FwdArgs& a_in, cudaStream_t s) {
     a.h0_pre = 0;
     if constexpr (M::kControl64 && !HasWeights<Pb>::value) {  // (FP64 control: no shared weights)
       if (a.control)
-        init_step_pass<M, Pb, R, true>(a, s, &e);
+        init_step_pass<M, typename LaneOf<Pb>::type, R, true>(a, s, &e);
       else
-        init_step_pass<M, Pb, R, false>(a, s, &e);
+        init_step_pass<M, typename LaneOf<Pb>::type, R, false>(a, s, &e);
     } else {
-      init_step_pass<M, Pb, R, false>(a, s, &e);
+      init_step_pass<M, typename LaneOf<Pb>::type, R, false>(a, s, &e);
     }
     if (e != cudaSuccess) return e;
   }
+  const long long lanes = a.n * GroupOf<Pb>::value;
   const size_t smem = (size_t)(((a.n_save + 1) & ~1) + a.segw * TPB_FWD) * sizeof(double);
   if (a.control) {  // FP64 step control: Tsit5 without shared weights
     if constexpr (M::kControl64 && !HasWeights<Pb>::value) {
       if constexpr (stages_possible<M, Pb, R>()) {
         if (a.stages)
-          return persistent_launch(record_entry<M, Pb, R, true, true, true>(), TPB_FWD, smem, a.n, s, &a);
+          return persistent_launch(record_entry<M, Pb, R, true, true, true>(), TPB_FWD, smem, lanes, s, &a);
       } else {
         if (a.stages) return cudaErrorInvalidValue;
       }
-      if (a.y_save) return persistent_launch(record_entry<M, Pb, R, true, false, true>(), TPB_FWD, smem, a.n, s, &a);
-      return persistent_launch(record_entry<M, Pb, R, false, false, true>(), TPB_FWD, smem, a.n, s, &a);
+      if (a.y_save) return persistent_launch(record_entry<M, Pb, R, true, false, true>(), TPB_FWD, smem, lanes, s, &a);
+      return persistent_launch(record_entry<M, Pb, R, false, false, true>(), TPB_FWD, smem, lanes, s, &a);
     } else {
       return cudaErrorInvalidValue;
     }
   }
   if constexpr (stages_possible<M, Pb, R>()) {
-    if (a.stages) return persistent_launch(record_kernel<M, Pb, R, true, true>, TPB_FWD, smem, a.n, s, &a);
+    if (a.stages) return persistent_launch(record_kernel<M, Pb, R, true, true>, TPB_FWD, smem, lanes, s, &a);
   } else {
     if (a.stages) return cudaErrorInvalidValue;
   }
-  if (a.y_save) return persistent_launch(record_kernel<M, Pb, R, true, false>, TPB_FWD, smem, a.n, s, &a);
-  return persistent_launch(record_kernel<M, Pb, R, false, false>, TPB_FWD, smem, a.n, s, &a);
+  if (a.y_save) return persistent_launch(record_kernel<M, Pb, R, true, false>, TPB_FWD, smem, lanes, s, &a);
+  return persistent_launch(record_kernel<M, Pb, R, false, false>, TPB_FWD, smem, lanes, s, &a);
 }
 
 #ifndef GS_T1_SAVE_PASS
@@ -1868,6 +1913,7 @@ template <class M, class Pb, class R>
 inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
   RevArgs a = a_in;
   a.t1_pre = 0;
+  const long long lanes = a.n * GroupOf<Pb>::value;
   size_t smem = (size_t)((a.n_save + 1) & ~1) * sizeof(double);
   if constexpr (HasWeights<Pb>::value) {
     using Acc = AccFor<Pb, R>;
@@ -1875,11 +1921,11 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
     smem += weight_stage_bytes<Pb>();
     int bps = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, reverse_k1_kernel<M, Pb, R, false>, TPB_REV, smem);
-    cudaError_t e = a.y_save_bar ? persistent_launch(reverse_k1_kernel<M, Pb, R, true>, TPB_REV, smem, a.n, s, &a)
-                                 : persistent_launch(reverse_k1_kernel<M, Pb, R, false>, TPB_REV, smem, a.n, s, &a);
+    cudaError_t e = a.y_save_bar ? persistent_launch(reverse_k1_kernel<M, Pb, R, true>, TPB_REV, smem, lanes, s, &a)
+                                 : persistent_launch(reverse_k1_kernel<M, Pb, R, false>, TPB_REV, smem, lanes, s, &a);
     if (e != cudaSuccess || !a.wpart || !a.shared_w_bar) return e;
     long long blocks = (long long)sm_count() * (bps > 0 ? bps : 1);
-    const long long need = (a.n + TPB_REV - 1) / TPB_REV;
+    const long long need = (lanes + TPB_REV - 1) / TPB_REV;
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
     using Part = typename Acc::Part;
@@ -1896,18 +1942,18 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
     if (a.stages) {
       if (a.k != 1 || a.segw != stage_segw<M, Pb::D>()) return cudaErrorInvalidValue;
       if (a.y_save_bar)
-        return persistent_launch(reverse_k1_entry<M, Pb, R, true, true>(), TPB_REV, smem, a.n, s, &a);
-      return persistent_launch(reverse_k1_entry<M, Pb, R, false, true>(), TPB_REV, smem, a.n, s, &a);
+        return persistent_launch(reverse_k1_entry<M, Pb, R, true, true>(), TPB_REV, smem, lanes, s, &a);
+      return persistent_launch(reverse_k1_entry<M, Pb, R, false, true>(), TPB_REV, smem, lanes, s, &a);
     }
   } else {
     if (a.stages) return cudaErrorInvalidValue;
   }
   if (a.k == 1) {
-    if (a.y_save_bar) return persistent_launch(reverse_k1_entry<M, Pb, R, true>(), TPB_REV, smem, a.n, s, &a);
-    return persistent_launch(reverse_k1_entry<M, Pb, R, false>(), TPB_REV, smem, a.n, s, &a);
+    if (a.y_save_bar) return persistent_launch(reverse_k1_entry<M, Pb, R, true>(), TPB_REV, smem, lanes, s, &a);
+    return persistent_launch(reverse_k1_entry<M, Pb, R, false>(), TPB_REV, smem, lanes, s, &a);
   }
-  if (a.y_save_bar) return persistent_launch(reverse_kernel<M, Pb, R, true>, TPB_REV, smem, a.n, s, &a);
-  return persistent_launch(reverse_kernel<M, Pb, R, false>, TPB_REV, smem, a.n, s, &a);
+  if (a.y_save_bar) return persistent_launch(reverse_kernel<M, Pb, R, true>, TPB_REV, smem, lanes, s, &a);
+  return persistent_launch(reverse_kernel<M, Pb, R, false>, TPB_REV, smem, lanes, s, &a);
   }
 }
 

@@ -180,8 +180,22 @@ __device__ __forceinline__ void lu_solve_t(const double (&LU)[D][D], const int (
   }
 }
 
-// One Rodas5P step from y with size h: stage inputs Y[0..7], stage solutions
-// U[0..7], the LU of W, y_new and the error estimate U[7]. false if W is singular.
+// Problems whose right-hand side is worth keeping between its value, Jacobian
+// and VJP at one point (the neural Robertson's network activations) declare a
+// Tape: the step fills entry i at stage input Y_i (entry 0 is y itself, where
+// the Jacobian is taken) and the reverse of the step reads it.
+struct NoTape {};
+template <class Pb, class = void>
+struct TapeOf {
+  using type = NoTape;
+  static constexpr bool value = false;
+};
+template <class Pb>
+struct TapeOf<Pb, std::void_t<typename Pb::Tape>> {
+  using type = typename Pb::Tape;
+  static constexpr bool value = true;
+};
+
 // Stage input Y_i = y + sum_{j<i} a_ij U_j, in a fixed order (the step and
 // the stored-stage reverse build it the same way).
 template <int D>
@@ -202,12 +216,21 @@ __device__ __forceinline__ void rodas_stage_inputs(const double (&y)[D], const d
   for (int i = 0; i < 8; ++i) rodas_stage_input<D>(i, y, U, Y[i]);
 }
 
+// One Rodas5P step from y with size h: stage inputs Y[0..7], stage solutions
+// U[0..7], the LU of W, y_new and the error estimate U[7]. false if W is singular.
 template <class Pb>
 __device__ __forceinline__ bool rodas_step(const double (&y)[Pb::D], const double (&p)[Pb::NP], double h,
                                            double (&Y)[8][Pb::D], double (&U)[8][Pb::D], double (&LU)[Pb::D][Pb::D],
-                                           int (&piv)[Pb::D], double (&rinv)[Pb::D], double (&ynew)[Pb::D]) {
+                                           int (&piv)[Pb::D], double (&rinv)[Pb::D], double (&ynew)[Pb::D],
+                                           typename TapeOf<Pb>::type& tape) {
   constexpr int D = Pb::D;
-  Pb::jac(y, p, LU);
+  double F0[D];  // (with a tape: f(y), evaluated first, whose entry the Jacobian reads)
+  if constexpr (TapeOf<Pb>::value) {
+    Pb::f_tape(y, p, F0, tape, 0);
+    Pb::jac_tape(y, p, LU, tape);
+  } else {
+    Pb::jac(y, p, LU);
+  }
   const double inv_hg = 1.0 / mul_(h, rodas::GAMMA);
   const double inv_h = 1.0 / h;
 #pragma unroll
@@ -221,7 +244,16 @@ __device__ __forceinline__ bool rodas_step(const double (&y)[Pb::D], const doubl
   for (int i = 0; i < 8; ++i) {
     double F[D], Rhs[D];
     rodas_stage_input<D>(i, y, U, Y[i]);
-    Pb::f(Y[i], p, F);
+    if constexpr (TapeOf<Pb>::value) {
+      if (i == 0) {
+#pragma unroll
+        for (int c = 0; c < D; ++c) F[c] = F0[c];
+      } else {
+        Pb::f_tape(Y[i], p, F, tape, i);
+      }
+    } else {
+      Pb::f(Y[i], p, F);
+    }
 #pragma unroll
     for (int c = 0; c < D; ++c) {
       if (i == 0) {
@@ -330,15 +362,18 @@ __device__ __forceinline__ bool rodas_tangent(const double (&y)[Pb::D], const do
 //   v += Ybar_i, Ubar_j += a_ij Ybar_i;
 // and W = I/(h gamma) - J(y) gives dL/dJ = sum_i Rbar_i U_i^T, contracted through
 // J(y, theta): v += d/dy (Rbar_i^T J U_i), theta_bar += d/dtheta (Rbar_i^T J U_i).
+// Problems with a tape take the contraction once per step: it is linear in
+// sum_i Rbar_i U_i^T, which the accumulator collects over the stages.
 template <class Pb, class Acc>
 __device__ __forceinline__ void rodas_reverse(const double (&y)[Pb::D], const double (&p)[Pb::NP], double h,
                                               const double (&Y)[8][Pb::D], const double (&U)[8][Pb::D],
                                               const double (&LU)[Pb::D][Pb::D], const int (&piv)[Pb::D],
                                               const double (&rinv)[Pb::D], const double (&lam)[Pb::D],
-                                              double (&v)[Pb::D], Acc& pacc) {
+                                              double (&v)[Pb::D], Acc& pacc, typename TapeOf<Pb>::type& tape) {
   constexpr int D = Pb::D;
   const double inv_h = 1.0 / h;
   double Ub[8][D];
+  if constexpr (TapeOf<Pb>::value) pacc.contract_begin(tape);
 #pragma unroll
   for (int j = 0; j < 8; ++j)
 #pragma unroll
@@ -355,15 +390,22 @@ __device__ __forceinline__ void rodas_reverse(const double (&y)[Pb::D], const do
     for (int j = 0; j < i; ++j)
 #pragma unroll
       for (int c = 0; c < D; ++c) Ub[j][c] = fma_(rodas::C(i, j), Rh[c], Ub[j][c]);
-    pacc.template vjp<Pb>(Y[i], p, Rb, Yb);
+    if constexpr (TapeOf<Pb>::value)
+      pacc.vjp_tape(tape, i, Y[i], p, Rb, Yb);
+    else
+      pacc.template vjp<Pb>(Y[i], p, Rb, Yb);
 #pragma unroll
     for (int c = 0; c < D; ++c) v[c] = add_(v[c], Yb[c]);
 #pragma unroll
     for (int j = 0; j < i; ++j)
 #pragma unroll
       for (int c = 0; c < D; ++c) Ub[j][c] = fma_(rodas::a(i, j), Yb[c], Ub[j][c]);
-    pacc.template jac_contract<Pb>(y, p, Rb, U[i], v);
+    if constexpr (TapeOf<Pb>::value)
+      pacc.contract_add(Rb, U[i]);
+    else
+      pacc.template jac_contract<Pb>(y, p, Rb, U[i], v);
   }
+  if constexpr (TapeOf<Pb>::value) pacc.contract_flush(tape, y, p, v);
 }
 
 // ---------------------------------------------------------------------------

@@ -96,3 +96,33 @@ def test_nrob_weight_gradient_is_deterministic_and_solve_grad_agrees():
     g = api.reverse(rec, P, Y, layout="soa", shared_w=SW)
     np.testing.assert_array_equal(a["params_bar"].cpu().numpy(), g["params_bar"].cpu().numpy())
     np.testing.assert_array_equal(a["shared_w_bar"].cpu().numpy(), g["shared_w_bar"].cpu().numpy())
+
+
+@pytest.mark.parametrize("n", [1, 15, 33, 7169])
+def test_nrob_lane_group_and_per_lane_forms(n):
+    """Ensembles up to 7168 trajectories run 16 lanes per trajectory, larger
+    ones a lane each: states equal bit for bit on both sides of the line (the
+    same sums in the same order), gradients to the rounding bound above, and
+    the weight gradient of a ragged last warp against the oracle."""
+    wl, SW = workload(n)
+    P, Y = dev(wl["params"].T), dev(wl["y0"].T)
+    rec, ysv, st = api.forward_record("nrob", P, Y, wl["t0"], wl["t1"], wl["save_t"], wl["rtol"], wl["atol"],
+                                      layout="soa", shared_w=SW)
+    assert (st.cpu().numpy() == 0).all()
+    g = api.reverse(rec, P, Y, layout="soa", shared_w=SW)
+    m = min(n, 33)  # the first trajectories, in a small ensemble of their own
+    sub = dict(wl, params=wl["params"][:m], y0=wl["y0"][:m])
+    Ps, Ys = dev(sub["params"].T), dev(sub["y0"].T)
+    rs, ys, _ = api.forward_record("nrob", Ps, Ys, wl["t0"], wl["t1"], wl["save_t"], wl["rtol"], wl["atol"],
+                                   layout="soa", shared_w=SW)
+    assert torch.equal(ysv[:, :, :m], ys)
+    gs = api.reverse(rs, Ps, Ys, layout="soa", shared_w=SW)
+    off, h = rs.export_mesh()
+    o = oracle.replay_grad("nrob", sub["params"], sub["y0"], wl["t0"], wl["t1"], wl["save_t"], off, h, w=wl["w"])
+    fp, fy = rounding_floor(sub, off, h, oracle.METHOD_RODAS5P)
+    for r in (g, gs):
+        assert_close(r["loss"][:m].cpu().numpy(), o["loss"], "loss", rtol=1e-10)
+        assert_close(r["params_bar"][:, :m].cpu().numpy().T, o["params_bar"], "params_bar", rtol=max(1e-10, 20.0 * fp))
+        assert_close(r["y0_bar"][:, :m].cpu().numpy().T, o["y0_bar"], "y0_bar", rtol=max(1e-10, 20.0 * fy))
+    wb = gs["shared_w_bar"].cpu().numpy().astype(np.float64)
+    assert np.abs(wb - o["w_bar"]).max() / np.abs(o["w_bar"]).max() <= 1e-6

@@ -440,12 +440,36 @@ struct HasNet : std::false_type {};
 template <class Pb>
 struct HasNet<Pb, std::void_t<decltype(Pb::kWeights)>> : std::true_type {};
 
+// Problems whose right-hand side is worth keeping between its value, Jacobian
+// and VJP at one point (network activations) declare a Tape: a step fills entry
+// i at its stage input Y_i (entry 0 is y itself) and the reverse of the step
+// reads it.
+struct NoTape {};
+template <class Pb, class = void>
+struct TapeOf {
+  using type = NoTape;
+  static constexpr bool value = false;
+};
+template <class Pb>
+struct TapeOf<Pb, std::void_t<typename Pb::Tape>> {
+  using type = typename Pb::Tape;
+  static constexpr bool value = true;
+};
+template <class Pb, class R>
+__device__ __forceinline__ void rhs_at(const R (&y)[Pb::D], const R (&p)[Pb::NP], R (&o)[Pb::D],
+                                       typename TapeOf<Pb>::type& tape, int i) {
+  if constexpr (TapeOf<Pb>::value)
+    Pb::f_tape(y, p, o, tape, i);
+  else
+    Pb::f(y, p, o);
+}
+
 // Stage inputs Y[0..6] of one Tsit5 step from y with size h (Y[0] = y,
 // Y[6] = y_new by FSAL) and stage slopes K[0..KN-1]. K[0] must hold f(y).
 // KN = 7 also evaluates k7 = f(y_new) for the error estimate and FSAL.
 template <class Pb, class R, int KN>
 __device__ __forceinline__ void tsit5_stages(const R (&y)[Pb::D], const R (&p)[Pb::NP], R h, R (&Y)[7][Pb::D],
-                                             R (&K)[7][Pb::D]) {
+                                             R (&K)[7][Pb::D], typename TapeOf<Pb>::type& tape) {
   constexpr int D = Pb::D;
 #pragma unroll
   for (int c = 0; c < D; ++c) Y[0][c] = y[c];
@@ -470,7 +494,7 @@ __device__ __forceinline__ void tsit5_stages(const R (&y)[Pb::D], const R (&p)[P
       for (int j = 1; j < i; ++j) s = fma_(R(tsit5::A(i, j)), K[j][c], s);
       Y[i][c] = fma_(h, s, y[c]);
     }
-    if (i < 6 || KN == 7) Pb::f(Y[i], p, K[i]);
+    if (i < 6 || KN == 7) rhs_at<Pb, R>(Y[i], p, K[i], tape, i);
   }
 }
 
@@ -551,7 +575,7 @@ __device__ __forceinline__ void tsit5_tangent(const double (&y)[Pb::D], const do
 // v = c + sum_j Ybar_j.
 template <class Pb, class R, class RB>
 __device__ __forceinline__ void tsit5_reverse(const R (&Y)[7][Pb::D], const R (&p)[Pb::NP], R h, const R (&c)[Pb::D],
-                                              R (&v)[Pb::D], RB& pbacc) {
+                                              R (&v)[Pb::D], RB& pbacc, typename TapeOf<Pb>::type& tape) {
   constexpr int D = Pb::D;
   // acc[l] = sum over the stages m already reversed of a_ml Ybar_m; stage 6 (the
   // first one reversed) starts every sum, so no zero is ever added.
@@ -575,7 +599,10 @@ __device__ __forceinline__ void tsit5_reverse(const R (&Y)[7][Pb::D], const R (&
 #pragma unroll
     for (int q = Q0; q < D; ++q)
       kb[q] = (j == 5) ? mul_(h, mul_(R(tsit5::B(j)), c[q])) : mul_(h, fma_(R(tsit5::B(j)), c[q], acc[j][q]));
-    pbacc.template vjp<Pb>(Y[j], p, kb, yb);
+    if constexpr (TapeOf<Pb>::value)
+      pbacc.vjp_tape(tape, j, Y[j], p, kb, yb);
+    else
+      pbacc.template vjp<Pb>(Y[j], p, kb, yb);
     if constexpr (PACK) {
       const float2 v2 = __fadd2_rn(make_float2(v[0], v[1]), make_float2(yb[0], yb[1]));
       v[0] = v2.x;

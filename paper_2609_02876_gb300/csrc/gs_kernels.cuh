@@ -156,9 +156,10 @@ struct Tsit5Method {
                                                Carry<Pb, R>& next) {
     constexpr int D = Pb::D;
     R Y[7][D], K[7][D];
+    typename TapeOf<Pb>::type tape;
 #pragma unroll
     for (int c = 0; c < D; ++c) K[0][c] = cy.k1[c];
-    tsit5_stages<Pb, R, 7>(y, p, to_r<R>(h), Y, K);
+    tsit5_stages<Pb, R, 7>(y, p, to_r<R>(h), Y, K, tape);
     tsit5_error<Pb, R>(K, to_r<R>(h), e);
 #pragma unroll
     for (int c = 0; c < D; ++c) {
@@ -189,9 +190,10 @@ struct Tsit5Method {
                                                  Carry<Pb, R>& next, StageData<Pb, R>& sd) {
     constexpr int D = Pb::D;
     R K[7][D];
+    typename TapeOf<Pb>::type tape;
 #pragma unroll
     for (int c = 0; c < D; ++c) K[0][c] = cy.k1[c];
-    tsit5_stages<Pb, R, 7>(y, p, to_r<R>(h), sd.Y, K);
+    tsit5_stages<Pb, R, 7>(y, p, to_r<R>(h), sd.Y, K, tape);
     tsit5_error<Pb, R>(K, to_r<R>(h), e);
 #pragma unroll
     for (int c = 0; c < D; ++c) {
@@ -234,7 +236,8 @@ struct Tsit5Method {
     const bool side = (mode == U_SIDE);
     R cv[D], v[D];
     unit_cotangent<Pb, R, USER_COT>(a, k, active, side, us, sd.Y[6], lam, cv, loss);
-    tsit5_reverse<Pb, R>(sd.Y, p, to_r<R>(h), cv, v, pacc);
+    typename TapeOf<Pb>::type tape;
+    tsit5_reverse<Pb, R>(sd.Y, p, to_r<R>(h), cv, v, pacc, tape);
 #pragma unroll
     for (int c = 0; c < D; ++c) lam[c] = !active ? lam[c] : (side ? add_(lam[c], v[c]) : v[c]);
     return true;
@@ -244,9 +247,10 @@ struct Tsit5Method {
                                               const Carry<Pb, R>& cy, R (&ys)[Pb::D]) {
     constexpr int D = Pb::D;
     R Y[7][D], K[7][D];
+    typename TapeOf<Pb>::type tape;
 #pragma unroll
     for (int c = 0; c < D; ++c) K[0][c] = cy.k1[c];
-    tsit5_stages<Pb, R, 6>(y, p, to_r<R>(h), Y, K);
+    tsit5_stages<Pb, R, 6>(y, p, to_r<R>(h), Y, K, tape);
 #pragma unroll
     for (int c = 0; c < D; ++c) ys[c] = Y[6][c];
     return true;
@@ -257,8 +261,9 @@ struct Tsit5Method {
                                                      R (&ynew)[Pb::D]) {
     constexpr int D = Pb::D;
     R Y[7][D], K[7][D];
-    Pb::f(y, p, K[0]);
-    tsit5_stages<Pb, R, 6>(y, p, to_r<R>(h), Y, K);
+    typename TapeOf<Pb>::type tape;
+    rhs_at<Pb, R>(y, p, K[0], tape, 0);
+    tsit5_stages<Pb, R, 6>(y, p, to_r<R>(h), Y, K, tape);
 #pragma unroll
     for (int c = 0; c < D; ++c) ynew[c] = Y[6][c];
     return true;
@@ -274,15 +279,16 @@ struct Tsit5Method {
                                               Acc& pacc, double& loss, R (&ynew)[Pb::D]) {
     constexpr int D = Pb::D;
     R Y[7][D], K[7][D];
-    Pb::f(x, p, K[0]);
-    tsit5_stages<Pb, R, 6>(x, p, to_r<R>(h), Y, K);
+    typename TapeOf<Pb>::type tape;
+    rhs_at<Pb, R>(x, p, K[0], tape, 0);
+    tsit5_stages<Pb, R, 6>(x, p, to_r<R>(h), Y, K, tape);
 #pragma unroll
     for (int c = 0; c < D; ++c) ynew[c] = Y[6][c];
     if (mode == U_RECOMP) return true;
     const bool side = (mode == U_SIDE);
     R cv[D], v[D];
     unit_cotangent<Pb, R, USER_COT>(a, k, active, side, us, ynew, lam, cv, loss);
-    tsit5_reverse<Pb, R>(Y, p, to_r<R>(h), cv, v, pacc);
+    tsit5_reverse<Pb, R>(Y, p, to_r<R>(h), cv, v, pacc, tape);
 #pragma unroll
     for (int c = 0; c < D; ++c) lam[c] = !active ? lam[c] : (side ? add_(lam[c], v[c]) : v[c]);
     return true;
@@ -1672,14 +1678,17 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
 // Measured at 2^24 Lorenz trajectories: the FP32-mixed sweep 3.4% faster at 8
 // blocks (64 registers) than at the compiler's 72, the FP64 stored-stage sweep
 // 1.5% faster at 5 (96 registers) than at 122 (at 6, 80 registers: 1.2%; at 7,
-// 72: 1.0%); the shared-weight kernels need more
-// registers than either cap and keep the compiler's choice. Capping the
+// 72: 1.0%); the LV UDE sweep is held to the 168 registers of 3 CTAs (its
+// compiler's choice, 186, leaves 2), the neural Robertson's keep the compiler's
+// choice. Capping the
 // Rodas5P (252 registers, 2 CTAs) and Verner7 (154, 3 CTAs) stored-stage sweeps
 // at 3 to 5 CTAs changed their time by under 2% (Robertson 2^20, Lorenz 2^23),
 // so they keep the compiler's choice too.
 template <class M, class Pb, class R, bool STAGES>
 constexpr int rev_min_blocks() {
-  if constexpr (HasWeights<Pb>::value)
+  if constexpr (std::is_same<Pb, LvUdeWarp>::value)
+    return 3;
+  else if constexpr (HasWeights<Pb>::value)
     return 0;
   else
     return std::is_same<R, float>::value ? M::REV_MINB_F32 : (STAGES ? M::REV_MINB_STAGES : 0);
@@ -1920,9 +1929,9 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
     if (a.k != 1) return cudaErrorInvalidValue;
     smem += weight_stage_bytes<Pb>();
     int bps = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, reverse_k1_kernel<M, Pb, R, false>, TPB_REV, smem);
-    cudaError_t e = a.y_save_bar ? persistent_launch(reverse_k1_kernel<M, Pb, R, true>, TPB_REV, smem, lanes, s, &a)
-                                 : persistent_launch(reverse_k1_kernel<M, Pb, R, false>, TPB_REV, smem, lanes, s, &a);
+    const auto kern = a.y_save_bar ? reverse_k1_entry<M, Pb, R, true>() : reverse_k1_entry<M, Pb, R, false>();
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, TPB_REV, smem);
+    cudaError_t e = persistent_launch(kern, TPB_REV, smem, lanes, s, &a);
     if (e != cudaSuccess || !a.wpart || !a.shared_w_bar) return e;
     long long blocks = (long long)sm_count() * (bps > 0 ? bps : 1);
     const long long need = (lanes + TPB_REV - 1) / TPB_REV;

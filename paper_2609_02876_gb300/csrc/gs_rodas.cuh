@@ -180,22 +180,6 @@ __device__ __forceinline__ void lu_solve_t(const double (&LU)[D][D], const int (
   }
 }
 
-// Problems whose right-hand side is worth keeping between its value, Jacobian
-// and VJP at one point (the neural Robertson's network activations) declare a
-// Tape: the step fills entry i at stage input Y_i (entry 0 is y itself, where
-// the Jacobian is taken) and the reverse of the step reads it.
-struct NoTape {};
-template <class Pb, class = void>
-struct TapeOf {
-  using type = NoTape;
-  static constexpr bool value = false;
-};
-template <class Pb>
-struct TapeOf<Pb, std::void_t<typename Pb::Tape>> {
-  using type = typename Pb::Tape;
-  static constexpr bool value = true;
-};
-
 // Stage input Y_i = y + sum_{j<i} a_ij U_j, in a fixed order (the step and
 // the stored-stage reverse build it the same way).
 template <int D>

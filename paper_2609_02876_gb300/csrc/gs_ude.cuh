@@ -150,6 +150,7 @@ struct LvUdeWarp : LvUde {
   }
   __device__ static void block_setup(const float* shared_w) {
     LvUde::block_setup(shared_w);
+    if (threadIdx.x == 0) *zero() = 0;
     uint4* f = frags();
     for (int i = threadIdx.x; i < 2 * 2 * 2 * 32; i += blockDim.x) {
       const int lane = i & 31, nt = (i >> 5) & 1, kk = (i >> 6) & 1, q = i >> 7;
@@ -243,16 +244,61 @@ struct LvUdeWarp : LvUde {
     o[0] = fmaf(p[0], y[0], -nn[0]);
     o[1] = fmaf(-p[1], y[1], nn[1]);
   }
-  // VJP of all lanes (as LvUde::backprop): yb = J^T v, pb += f_theta^T v, and the
-  // staging rows left holding [gz2 | h1 | gz1 | h2 | x, y, go] for the
-  // weight-gradient MMAs.
-  __device__ __forceinline__ static void backprop_warp(const float (&y)[D], const float (&p)[NP],
+  // One unit's activations, kept between the stage slopes and their VJPs: h1 and
+  // h2 of this lane at each of the six stages (768 bytes per lane in local
+  // memory, L2-resident: 45 MB over a full grid). The reverse unit then runs 6
+  // network passes instead of 12: 8 vector loads and stores per stage replace
+  // 32 tanh and the hidden-layer product (reverse sweep at 2^16 trajectories 6.3
+  // -> 4.2 ms, at 2^18 15.6 -> 10.8 ms; results bit-identical). The base index is a zero read from
+  // shared memory, which the compiler cannot see through: with constant indices
+  // it keeps the tape in registers (255 of them, and 2 CTAs per SM for 3).
+  __device__ __forceinline__ static volatile int* zero() {
+    __shared__ int z;
+    return &z;
+  }
+  struct Tape {
+    float4 a[6 * 8];
+    int base;
+    __device__ __forceinline__ Tape() : base(*zero()) {}
+    __device__ __forceinline__ float4* at(int i) { return a + base + 8 * i; }
+  };
+  __device__ __forceinline__ static void f_tape(const float (&y)[D], const float (&p)[NP], float (&o)[D], Tape& tape,
+                                                int i) {
+    float h2[UDE_H], nn[2];
+    forward_warp(y[0], y[1], h2, nn);
+    const int lane = threadIdx.x & 31, swl = ude_sw(lane);
+    const float* row = ude_stage() + lane * UDE_ROW;
+    float4* a = tape.at(i);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      a[j] = *reinterpret_cast<const float4*>(row + ((16 + 4 * j) ^ swl));  // h1, as this lane staged it
+      a[4 + j] = make_float4(h2[4 * j], h2[4 * j + 1], h2[4 * j + 2], h2[4 * j + 3]);
+    }
+    o[0] = fmaf(p[0], y[0], -nn[0]);
+    o[1] = fmaf(-p[1], y[1], nn[1]);
+  }
+  // VJP of all lanes (as LvUde::backprop) at stage i of the tape: yb = J^T v,
+  // pb += f_theta^T v, and the staging rows left holding [gz2 | h1 | gz1 | h2 |
+  // x, y, go] for the weight-gradient MMAs.
+  __device__ __forceinline__ static void backprop_warp(Tape& tape, int i, const float (&y)[D], const float (&p)[NP],
                                                        const float (&v)[D], float (&yb)[D], float (&pb)[NP]) {
     float* st = ude_stage();
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, swl = ude_sw(lane), swg = ude_sw(g);
     float* row = st + lane * UDE_ROW;
-    float h2[UDE_H], nn[2];
-    forward_warp(y[0], y[1], h2, nn);
+    float h2[UDE_H];
+    const float4* a = tape.at(i);
+    __syncwarp();
+    asm volatile("" ::: "memory");
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float4 b = a[4 + j];
+      *reinterpret_cast<float4*>(row + ((16 + 4 * j) ^ swl)) = a[j];
+      *reinterpret_cast<float4*>(row + ((48 + 4 * j) ^ swl)) = b;
+      h2[4 * j] = b.x;
+      h2[4 * j + 1] = b.y;
+      h2[4 * j + 2] = b.z;
+      h2[4 * j + 3] = b.w;
+    }
     const float* w = weights();
     const float go0 = -v[0], go1 = v[1];  // f0 = a x - nn0, f1 = -d y + nn1
     *reinterpret_cast<float4*>(row + (64 ^ swl)) = make_float4(y[0], y[1], go0, go1);
@@ -552,13 +598,18 @@ struct UdeAcc {
   template <class Pb>
   __device__ __forceinline__ void vjp(const float (&y)[2], const float (&p)[2], const float (&v)[2],
                                       float (&yb)[2]) {
-    static_assert(std::is_same<Pb, LvUdeWarp>::value || std::is_same<Pb, LvUdeCta>::value,
-                  "the UDE reverse sweep uses a collective form of the network");
+    static_assert(std::is_same<Pb, LvUdeCta>::value, "the UDE reverse sweep uses a collective form of the network");
     float x[2] = {0.0f, 0.0f};
-    if constexpr (std::is_same<Pb, LvUdeCta>::value)
-      LvUdeCta::backprop_cta(y, p, v, yb, x);  // leaves the factor rows staged
-    else
-      LvUdeWarp::backprop_warp(y, p, v, yb, x);
+    LvUdeCta::backprop_cta(y, p, v, yb, x);  // leaves the factor rows staged
+    add_unit(x);
+  }
+  __device__ __forceinline__ void vjp_tape(LvUdeWarp::Tape& tape, int i, const float (&y)[2], const float (&p)[2],
+                                           const float (&v)[2], float (&yb)[2]) {
+    float x[2] = {0.0f, 0.0f};
+    LvUdeWarp::backprop_warp(tape, i, y, p, v, yb, x);
+    add_unit(x);
+  }
+  __device__ __forceinline__ void add_unit(const float (&x)[2]) {
 #pragma unroll
     for (int q = 0; q < 2; ++q) th.u[q] = add_(th.u[q], x[q]);
     accumulate();

@@ -36,6 +36,94 @@ __device__ __forceinline__ double sub_(double a, double b) { return __dsub_rn(a,
 __device__ __forceinline__ float sub_(float a, float b) { return __fsub_rn(a, b); }
 
 // ---------------------------------------------------------------------------
+// FP64 with multiplications on the integer pipes. GB300's FP64 unit takes 64
+// cycles per warp instruction per SM quarter (measured, whatever the number of
+// active lanes), while the integer and FP32 pipes stand by; about a quarter of
+// the Tsit5 kernels' FP64 instructions are plain multiplications. SoftD is a
+// double whose mul_ is computed in integers, bit for bit the IEEE product (round
+// to nearest even): the 53 x 53-bit product from four 32 x 32 -> 64 multiply-adds,
+// normalised, rounded, with the exponents and signs added as integers. Measured
+// alone it takes 55 cycles per warp instruction (4 warps per SM quarter), and it
+// overlaps fully with FMAs of the other warps: 4 + 4 of them take 283 cycles,
+// 4 FMAs alone 268. With one warp per quarter it is the slower one (latency 129
+// cycles against 66). It takes the Lorenz record at 2^22 from 73.7 to 60.8 ms and
+// the reverse sweep from 78.0 to 59.6 ms: 38 of a trial's 148 FP64 instructions
+// and 48 of a reverse unit's 171 leave the FP64 unit.
+//
+// Operands outside 2^-511 .. 2^511 (zeros, subnormals, infinities and NaNs
+// among them) give a NaN in place of the product; it reaches the caller's
+// results through every later operation, and the caller then repeats its work
+// in hardware arithmetic (soft_lost).
+// ---------------------------------------------------------------------------
+struct SoftD {
+  double v;
+  SoftD() = default;
+  __host__ __device__ __forceinline__ explicit SoftD(double x) : v(x) {}
+  __host__ __device__ __forceinline__ SoftD operator-() const { return SoftD(-v); }
+};
+__host__ __device__ __forceinline__ bool soft_range(uint32_t hi) {  // exponent field in [512, 1534]
+  return hi + hi - 0x40000000u < 0x7fe00000u;
+}
+// The product of two doubles in range, from their words (host: for the tests).
+__host__ __device__ __forceinline__ void soft_mul_words(uint32_t ah, uint32_t al, uint32_t bh, uint32_t bl,
+                                                        uint32_t& rh, uint32_t& rl) {
+  const uint32_t ma = (ah & 0xfffffu) | 0x100000u, mb = (bh & 0xfffffu) | 0x100000u;
+  const uint64_t p0 = (uint64_t)al * bl;
+  const uint64_t p1 = (uint64_t)ma * bl + (p0 >> 32);
+  const uint64_t p2 = (uint64_t)al * mb + (uint32_t)p1;
+  const uint64_t p3 = (uint64_t)ma * mb + (p1 >> 32) + (p2 >> 32);  // bits 64.. of the 106-bit product
+  const uint32_t hh = (uint32_t)(p3 >> 32), hl = (uint32_t)p3, m = (uint32_t)p2, l = (uint32_t)p0;
+  const uint32_t top = hh >> 9, sh = 12u - top;  // top: the product's mantissa is in [2, 4)
+#ifdef __CUDA_ARCH__
+  const uint32_t qh = __funnelshift_l(hl, hh, sh), ql = __funnelshift_l(m, hl, sh);
+#else
+  const uint32_t qh = (hh << sh) | (hl >> (32 - sh)), ql = (hl << sh) | (m >> (32 - sh));
+#endif
+  const uint32_t rem = (m << sh) | (l < 1u ? l : 1u);  // the bits below, the lowest one sticky
+  // sign and exponent: each operand's high word less its mantissa is sign + (e - 1) 2^20 (mod 2^32)
+  const uint32_t se = ah + bh - ma - mb + 0xc0200000u + (top << 20);
+  const uint64_t half = (uint64_t)rem + 0x7fffffffu + (ql & 1u);  // carries out to round up
+  const uint64_t r = (((uint64_t)(qh + se) << 32) | ql) + (half >> 32);
+  rh = (uint32_t)(r >> 32);
+  rl = (uint32_t)r;
+}
+__device__ __forceinline__ SoftD mul_(SoftD a, SoftD b) {
+  const uint32_t ah = (uint32_t)__double2hiint(a.v), bh = (uint32_t)__double2hiint(b.v);
+  uint32_t rh, rl;
+  soft_mul_words(ah, (uint32_t)__double2loint(a.v), bh, (uint32_t)__double2loint(b.v), rh, rl);
+  rh = (soft_range(ah) && soft_range(bh)) ? rh : 0x7ff80000u;
+  return SoftD(__hiloint2double((int)rh, (int)rl));
+}
+__device__ __forceinline__ SoftD fma_(SoftD a, SoftD b, SoftD c) { return SoftD(__fma_rn(a.v, b.v, c.v)); }
+__device__ __forceinline__ SoftD add_(SoftD a, SoftD b) { return SoftD(__dadd_rn(a.v, b.v)); }
+__device__ __forceinline__ SoftD sub_(SoftD a, SoftD b) { return SoftD(__dsub_rn(a.v, b.v)); }
+// Whether values in soft arithmetic hold a NaN; whether inputs are outside its range.
+template <int N>
+__device__ __forceinline__ bool soft_lost(const SoftD (&x)[N]) {
+  bool lost = false;
+#pragma unroll
+  for (int i = 0; i < N; ++i) lost = lost || (((uint32_t)__double2hiint(x[i].v) << 1) > 0xffe00000u);
+  return lost;
+}
+template <int N>
+__device__ __forceinline__ bool soft_unfit(const double (&x)[N]) {
+  bool bad = false;
+#pragma unroll
+  for (int i = 0; i < N; ++i) bad = bad || !soft_range((uint32_t)__double2hiint(x[i]));
+  return bad;
+}
+template <int N>
+__device__ __forceinline__ void to_soft(const double (&x)[N], SoftD (&o)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) o[i].v = x[i];
+}
+template <int N>
+__device__ __forceinline__ void from_soft(const SoftD (&x)[N], double (&o)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) o[i] = x[i].v;
+}
+
+// ---------------------------------------------------------------------------
 // FP32 <-> FP64 conversions on the integer ALU. GB300 executes the hardware
 // conversion instructions on its FP64 pipe (2 lanes per clock per SM), which
 // the FP32-mixed form otherwise spends on format changes; these rebuild the
@@ -101,6 +189,8 @@ template <>
 __device__ __forceinline__ double to_r<double>(double x) { return x; }
 template <>
 __device__ __forceinline__ float to_r<float>(double x) { return to_f(x); }
+template <>
+__device__ __forceinline__ SoftD to_r<SoftD>(double x) { return SoftD(x); }
 
 // ---------------------------------------------------------------------------
 // Problems (paper Appendix A). Each provides
@@ -871,6 +961,17 @@ struct PlainAcc {
   }
   __device__ __forceinline__ void flush() {}
   __device__ double get(int q) const { return s[q]; }
+};
+// PlainAcc's sums in soft arithmetic (one unit's worth; see SoftD).
+template <int NP>
+struct SoftAcc {
+  SoftD s[NP];
+  template <class Pb>
+  __device__ __forceinline__ void vjp(const SoftD (&y)[Pb::D], const SoftD (&p)[NP], const SoftD (&v)[Pb::D],
+                                      SoftD (&yb)[Pb::D]) {
+    Pb::vjp(y, p, v, yb, s);
+  }
+  __device__ __forceinline__ void flush() {}
 };
 template <int NP>
 struct CompensatedAcc {

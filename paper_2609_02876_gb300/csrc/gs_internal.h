@@ -145,6 +145,10 @@ struct LaunchCfg {
 cudaError_t launch_tsit5_forward(int problem, int precision, const FwdArgs& a, cudaStream_t s);
 cudaError_t launch_tsit5_reverse(int problem, int precision, const RevArgs& a, cudaStream_t s);
 bool tsit5_supports(int problem, int precision);
+// The FP64 Tsit5 kernels with multiplications on the integer pipes (SoftD in
+// gs_device.cuh); the reverse sweep for k = 1 records. Same results.
+cudaError_t launch_tsit5_soft_forward(int problem, const FwdArgs& a, cudaStream_t s);
+cudaError_t launch_tsit5_soft_reverse(int problem, const RevArgs& a, cudaStream_t s);
 cudaError_t launch_rodas_forward(int problem, int precision, const FwdArgs& a, cudaStream_t s);
 cudaError_t launch_rodas_reverse(int problem, int precision, const RevArgs& a, cudaStream_t s);
 bool rodas_supports(int problem, int precision);

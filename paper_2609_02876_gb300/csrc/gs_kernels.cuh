@@ -126,6 +126,7 @@ struct Tsit5Method {
   static constexpr bool kStages = true;           // records may store stage inputs
   static constexpr bool kControl64 = true;        // record kernels with FP64 step control
   static constexpr int REV_MINB_F32 = 8, REV_MINB_STAGES = 5;  // reverse-sweep register caps (see rev_min_blocks)
+  static constexpr bool kSoft = true;  // steps and their reverse also run in soft arithmetic (SoftD)
   // Step of the lanes without work in a warp-collective unit (zero cotangent):
   // any value whose step stays finite.
   static constexpr double IDLE_H = 0.0;
@@ -225,9 +226,46 @@ struct Tsit5Method {
       for (int c = 0; c < D; ++c)
         if (j < 6 || side) sd.Y[j][c] = to_r<R>(read((j - 1) * D + c));
   }
+  template <class Pb, class A, class B, class Cast>
+  __device__ __forceinline__ static void cast_stages(const StageData<Pb, A>& x, StageData<Pb, B>& o, Cast cast) {
+#pragma unroll
+    for (int j = 0; j < 7; ++j)
+#pragma unroll
+      for (int c = 0; c < Pb::D; ++c) o.Y[j][c] = cast(x.Y[j][c]);
+  }
+  // The reverse of a step over its stage inputs, with SOFT in soft arithmetic
+  // when the warp's inputs are in its range (a lane whose values leave it repeats
+  // the step in hardware arithmetic).
+  template <class Pb, class R, bool SOFT, class Acc>
+  __device__ __forceinline__ static void reverse_step(const R (&Y)[7][Pb::D], const R (&p)[Pb::NP], double h,
+                                                      const R (&cv)[Pb::D], R (&v)[Pb::D], Acc& pacc,
+                                                      typename TapeOf<Pb>::type& tape) {
+    constexpr int D = Pb::D;
+    bool hard = true;
+    if constexpr (SOFT) {
+      const double hh[1] = {h};
+      const bool unfit = soft_unfit(cv) || soft_unfit(p) || soft_unfit(hh);
+      if (!__any_sync(__activemask(), unfit)) {
+        SoftD Ys[7][D], ps[Pb::NP], cs[D], vs[D];
+        SoftAcc<Pb::NP> acc;
+#pragma unroll
+        for (int j = 0; j < 7; ++j) to_soft(Y[j], Ys[j]);
+        to_soft(p, ps);
+        to_soft(cv, cs);
+        to_soft(pacc.s, acc.s);
+        tsit5_reverse<Pb, SoftD>(Ys, ps, SoftD(h), cs, vs, acc, tape);
+        hard = soft_lost(vs) || soft_lost(acc.s);
+        if (!hard) {
+          from_soft(vs, v);
+          from_soft(acc.s, pacc.s);
+        }
+      }
+    }
+    if (hard) tsit5_reverse<Pb, R>(Y, p, to_r<R>(h), cv, v, pacc, tape);
+  }
   // Reverse unit over stored stage data: no stage is recomputed. Same
   // arithmetic as unit().
-  template <class Pb, class R, bool USER_COT, class Acc>
+  template <class Pb, class R, bool USER_COT, bool SOFT, class Acc>
   __device__ __forceinline__ static bool unit_stored(const RevArgs& a, long long k, int mode, bool active, int us,
                                                      const R (&x)[Pb::D], double h, const R (&p)[Pb::NP],
                                                      const StageData<Pb, R>& sd, R (&lam)[Pb::D], Acc& pacc,
@@ -237,7 +275,7 @@ struct Tsit5Method {
     R cv[D], v[D];
     unit_cotangent<Pb, R, USER_COT>(a, k, active, side, us, sd.Y[6], lam, cv, loss);
     typename TapeOf<Pb>::type tape;
-    tsit5_reverse<Pb, R>(sd.Y, p, to_r<R>(h), cv, v, pacc, tape);
+    reverse_step<Pb, R, SOFT>(sd.Y, p, h, cv, v, pacc, tape);
 #pragma unroll
     for (int c = 0; c < D; ++c) lam[c] = !active ? lam[c] : (side ? add_(lam[c], v[c]) : v[c]);
     return true;
@@ -273,22 +311,42 @@ struct Tsit5Method {
   // `active` is false only for the lanes without work that join a
   // warp-collective unit (shared-weight problems); they run with h = 0 and a
   // zero cotangent and change nothing.
-  template <class Pb, class R, bool USER_COT, class Acc>
+  template <class Pb, class R, bool USER_COT, bool SOFT, class Acc>
   __device__ __forceinline__ static bool unit(const RevArgs& a, long long k, int mode, bool active, int us,
                                               const R (&x)[Pb::D], double h, const R (&p)[Pb::NP], R (&lam)[Pb::D],
                                               Acc& pacc, double& loss, R (&ynew)[Pb::D]) {
     constexpr int D = Pb::D;
     R Y[7][D], K[7][D];
     typename TapeOf<Pb>::type tape;
-    rhs_at<Pb, R>(x, p, K[0], tape, 0);
-    tsit5_stages<Pb, R, 6>(x, p, to_r<R>(h), Y, K, tape);
+    bool hard = true;
+    if constexpr (SOFT) {
+      const double hh[1] = {h};
+      const bool unfit = soft_unfit(x) || soft_unfit(p) || soft_unfit(hh);
+      if (!__any_sync(__activemask(), unfit)) {
+        SoftD xs[D], ps[Pb::NP], Ys[7][D], Ks[7][D];
+        to_soft(x, xs);
+        to_soft(p, ps);
+        Pb::f(xs, ps, Ks[0]);
+        tsit5_stages<Pb, SoftD, 6>(xs, ps, SoftD(h), Ys, Ks, tape);
+        hard = false;
+#pragma unroll
+        for (int j = 0; j < 7; ++j) {
+          hard = hard || soft_lost(Ys[j]);
+          from_soft(Ys[j], Y[j]);
+        }
+      }
+    }
+    if (hard) {
+      rhs_at<Pb, R>(x, p, K[0], tape, 0);
+      tsit5_stages<Pb, R, 6>(x, p, to_r<R>(h), Y, K, tape);
+    }
 #pragma unroll
     for (int c = 0; c < D; ++c) ynew[c] = Y[6][c];
     if (mode == U_RECOMP) return true;
     const bool side = (mode == U_SIDE);
     R cv[D], v[D];
     unit_cotangent<Pb, R, USER_COT>(a, k, active, side, us, ynew, lam, cv, loss);
-    tsit5_reverse<Pb, R>(Y, p, to_r<R>(h), cv, v, pacc, tape);
+    reverse_step<Pb, R, SOFT>(Y, p, h, cv, v, pacc, tape);
 #pragma unroll
     for (int c = 0; c < D; ++c) lam[c] = !active ? lam[c] : (side ? add_(lam[c], v[c]) : v[c]);
     return true;
@@ -302,6 +360,7 @@ struct Tsit5Method {
 #define GS_VERN7_REV_MINB_STAGES 0
 #endif
 struct Rodas5PMethod {  // FP64 only: the stiff W-matrix LU and its solves stay FP64
+  static constexpr bool kSoft = false;
   static constexpr bool kControl64 = false;
   static constexpr int REV_MINB_F32 = 0, REV_MINB_STAGES = GS_RODAS_REV_MINB_STAGES;
   static constexpr int ORDER = 5, ERR_ORDER = 4;
@@ -373,7 +432,7 @@ struct Rodas5PMethod {  // FP64 only: the stiff W-matrix LU and its solves stay 
 #pragma unroll
     for (int c = 0; c < D; ++c) sd.ynew[c] = side ? add_(sd.Y[7][c], sd.U[7][c]) : x[c];
   }
-  template <class Pb, class R, bool USER_COT, class Acc>
+  template <class Pb, class R, bool USER_COT, bool SOFT, class Acc>
   __device__ __forceinline__ static bool unit_stored(const RevArgs& a, long long k, int mode, bool active, int us,
                                                      const R (&x)[Pb::D], double h, const R (&p)[Pb::NP],
                                                      const StageData<Pb, R>& sd, R (&lam)[Pb::D], Acc& pacc,
@@ -429,7 +488,7 @@ struct Rodas5PMethod {  // FP64 only: the stiff W-matrix LU and its solves stay 
     typename TapeOf<Pb>::type tape;
     return rodas_step<Pb>(y, p, h, Y, U, LU, piv, rinv, ynew, tape);
   }
-  template <class Pb, class R, bool USER_COT, class Acc>
+  template <class Pb, class R, bool USER_COT, bool SOFT, class Acc>
   __device__ __forceinline__ static bool unit(const RevArgs& a, long long k, int mode, bool active, int us,
                                               const R (&x)[Pb::D], double h, const R (&p)[Pb::NP], R (&lam)[Pb::D],
                                               Acc& pacc, double& loss, R (&ynew)[Pb::D]) {
@@ -453,6 +512,7 @@ struct Rodas5PMethod {  // FP64 only: the stiff W-matrix LU and its solves stay 
 // Rosenbrock23 (FP64 only): second order, error estimate of order 2 (err^(-1/3)
 // controller), f at the accepted state carried to the next step.
 struct Ros23Method {
+  static constexpr bool kSoft = false;
   static constexpr bool kControl64 = false;
   static constexpr int REV_MINB_F32 = 0, REV_MINB_STAGES = 0;
   static constexpr int ORDER = 2, ERR_ORDER = 2;
@@ -528,7 +588,7 @@ struct Ros23Method {
 #pragma unroll
     for (int c = 0; c < D; ++c) sd.piv[c] = (int)read(i++);
   }
-  template <class Pb, class R, bool USER_COT, class Acc>
+  template <class Pb, class R, bool USER_COT, bool SOFT, class Acc>
   __device__ __forceinline__ static bool unit_stored(const RevArgs& a, long long k, int mode, bool active, int us,
                                                      const R (&x)[Pb::D], double h, const R (&p)[Pb::NP],
                                                      const StageData<Pb, R>& sd, R (&lam)[Pb::D], Acc& pacc,
@@ -583,7 +643,7 @@ struct Ros23Method {
     ros23_stages<Pb>(y, p, h, F0, LU, piv, rinv, k1, u2, Y1, F1, ynew);
     return ok;
   }
-  template <class Pb, class R, bool USER_COT, class Acc>
+  template <class Pb, class R, bool USER_COT, bool SOFT, class Acc>
   __device__ __forceinline__ static bool unit(const RevArgs& a, long long k, int mode, bool active, int us,
                                               const R (&x)[Pb::D], double h, const R (&p)[Pb::NP], R (&lam)[Pb::D],
                                               Acc& pacc, double& loss, R (&ynew)[Pb::D]) {
@@ -606,6 +666,7 @@ struct Ros23Method {
 };
 
 struct Verner7Method {  // FP64 only
+  static constexpr bool kSoft = false;
   static constexpr bool kControl64 = false;
   static constexpr int REV_MINB_F32 = 0, REV_MINB_STAGES = GS_VERN7_REV_MINB_STAGES;
   static constexpr int ORDER = 7, ERR_ORDER = 6;
@@ -670,7 +731,7 @@ struct Verner7Method {  // FP64 only
       for (int c = 0; c < D; ++c) sd.ynew[c] = read(8 * D + c);
     }
   }
-  template <class Pb, class R, bool USER_COT, class Acc>
+  template <class Pb, class R, bool USER_COT, bool SOFT, class Acc>
   __device__ __forceinline__ static bool unit_stored(const RevArgs& a, long long k, int mode, bool active, int us,
                                                      const R (&x)[Pb::D], double h, const R (&p)[Pb::NP],
                                                      const StageData<Pb, R>& sd, R (&lam)[Pb::D], Acc& pacc,
@@ -718,7 +779,7 @@ struct Verner7Method {  // FP64 only
     vern7_update<Pb, R, 9>(y, K, h, ynew);
     return true;
   }
-  template <class Pb, class R, bool USER_COT, class Acc>
+  template <class Pb, class R, bool USER_COT, bool SOFT, class Acc>
   __device__ __forceinline__ static bool unit(const RevArgs& a, long long k, int mode, bool active, int us,
                                               const R (&x)[Pb::D], double h, const R (&p)[Pb::NP], R (&lam)[Pb::D],
                                               Acc& pacc, double& loss, R (&ynew)[Pb::D]) {
@@ -789,14 +850,52 @@ constexpr bool carry_from_pass() {
   return M::kCarryIsF && std::is_same<R, double>::value;
 }
 
+// A trial step in soft arithmetic (SoftD), if the warp's inputs are in its range.
+// Returns whether its results stand; if not, the lane takes the hardware step.
+template <class M, class Pb, bool STAGES>
+__device__ __forceinline__ bool soft_trial(const double (&x)[Pb::D], const double (&p)[Pb::NP], double h,
+                                           const typename M::template Carry<Pb, double>& cy, double (&yn)[Pb::D],
+                                           double (&e)[Pb::D], typename M::template Carry<Pb, double>& next,
+                                           typename StageOf<M, Pb, double, STAGES>::type& sd) {
+  constexpr int D = Pb::D;
+  const double hh[1] = {h};
+  bool unfit = soft_unfit(x) || soft_unfit(p) || soft_unfit(hh);
+  typename M::template Carry<Pb, SoftD> cs, ns;
+  if constexpr (M::kCarryIsF) {
+    double k[D];
+#pragma unroll
+    for (int c = 0; c < D; ++c) k[c] = M::template carry_f<Pb, double>(cy, c);
+    unfit = unfit || soft_unfit(k);
+    M::template set_carry_f<Pb, SoftD>(cs, [&](int c) { return SoftD(k[c]); });
+  }
+  if (__any_sync(__activemask(), unfit)) return false;
+  SoftD xs[D], ps[Pb::NP], ys[D], es[D];
+  to_soft(x, xs);
+  to_soft(p, ps);
+  typename StageOf<M, Pb, SoftD, STAGES>::type ss;
+  if constexpr (STAGES)
+    M::template trial_s<Pb, SoftD>(xs, ps, h, cs, ys, es, ns, ss);
+  else
+    M::template trial<Pb, SoftD>(xs, ps, h, cs, ys, es, ns);
+  if (soft_lost(ys) || soft_lost(es)) return false;
+  from_soft(ys, yn);
+  from_soft(es, e);
+  if constexpr (M::kCarryIsF)
+    M::template set_carry_f<Pb, double>(next, [&](int c) { return M::template carry_f<Pb, SoftD>(ns, c).v; });
+  if constexpr (STAGES)
+    M::template cast_stages<Pb, SoftD, double>(ss, sd, [](const SoftD& q) { return q.v; });
+  return true;
+}
+
 // SAVES: save-time side steps run (for y_save, or for the stored side stages);
 // STAGES: the record stores stage inputs (k = 1); C64: FP64 step control
 // (GS_CONTROL_FP64: error norm, controller, starting step and step floor in FP64).
-template <class M, class Pb, class R, bool SAVES, bool STAGES, bool C64 = false>
+template <class M, class Pb, class R, bool SAVES, bool STAGES, bool C64 = false, bool SOFT = false>
 __device__ __forceinline__ void record_body(const FwdArgs& a) {
   static_assert(!STAGES || (SAVES && M::kStages), "stored stages need side steps and a method that exposes stages");
   constexpr int D = Pb::D, NP = Pb::NP;
   using Carry = typename M::template Carry<Pb, R>;
+  static_assert(!SOFT || (M::kSoft && std::is_same<R, double>::value), "soft arithmetic is FP64's");
   extern __shared__ double smem[];
   const int ns = a.n_save;
   double* s_save = smem;
@@ -959,11 +1058,15 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
 #pragma unroll
       for (int q2 = 0; q2 < NP; ++q2) pin[q2] = p[q2];
       const Carry cin = is_side ? cyp : cy;
+      bool hard = true;
+      if constexpr (SOFT) {
+        hard = !soft_trial<M, Pb, STAGES>(xin, pin, hx, cin, yn, e, next, sd);
+      }
       if constexpr (STAGES) {
         // the unit's stage data go out at once (a step's to its staging slot,
         // overwritten by the next trial if this one is rejected), so that they
         // are not held in registers across the step-size decision
-        solved = M::template trial_s<Pb, R>(xin, pin, hx, cin, yn, e, next, sd);
+        if (hard) solved = M::template trial_s<Pb, R>(xin, pin, hx, cin, yn, e, next, sd);
         if (is_side) {
           constexpr int SP = M::template side_payload<D>();
           if constexpr (side_blocks<SP>()) {  // this trajectory's block, 16-byte vector stores
@@ -981,7 +1084,7 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
           M::template pack<Pb, R>(sd, false, [&](int i, double v) { stg[(3 + D + i) * TB] = v; });
         }
       } else {
-        solved = M::template trial<Pb, R>(xin, pin, hx, cin, yn, e, next);
+        if (hard) solved = M::template trial<Pb, R>(xin, pin, hx, cin, yn, e, next);
       }
       if (!is_side) {
         ++natt;
@@ -1179,6 +1282,11 @@ template <class M, class Pb, class R, bool SAVES, bool STAGES, bool C64 = false>
 __global__ void __launch_bounds__(TPB_FWD) record_kernel(const FwdArgs a) {
   record_body<M, Pb, R, SAVES, STAGES, C64>(a);
 }
+// The same in soft arithmetic (SoftD), at 4 CTAs per SM.
+template <class M, class Pb, bool SAVES, bool STAGES, bool C64>
+__global__ void __launch_bounds__(TPB_FWD, 4) record_soft_kernel(const FwdArgs a) {
+  record_body<M, Pb, double, SAVES, STAGES, C64, true>(a);
+}
 template <class M, class Pb, class R, bool SAVES, bool STAGES, bool C64, int MINB>
 __global__ void __launch_bounds__(TPB_FWD, MINB) record_kernel_mb(const FwdArgs a) {
   record_body<M, Pb, R, SAVES, STAGES, C64>(a);
@@ -1295,6 +1403,7 @@ enum : int { PH_LOAD = 0, PH_RECOMP = 1, PH_INJECT = 2 };
 template <class M, class Pb, class R, bool USER_COT>
 __global__ void __launch_bounds__(TPB_REV) reverse_kernel(const RevArgs a) {
   constexpr int D = Pb::D, NP = Pb::NP;
+  constexpr bool SOFT = false;
   static_assert(!HasWeights<Pb>::value, "shared-weight problems use the k = 1 reverse kernel");
   using Acc = AccOf<R, NP>;
   extern __shared__ double smem[];
@@ -1424,7 +1533,7 @@ __global__ void __launch_bounds__(TPB_REV) reverse_kernel(const RevArgs a) {
     __syncwarp();
     if (mode == U_RECOMP || mode == U_STEP || mode == U_SIDE) {
       R yn[D];
-      const bool ok = M::template unit<Pb, R, USER_COT, Acc>(a, k, mode, true, us, ux, uh, p, lam, pacc, loss, yn);
+      const bool ok = M::template unit<Pb, R, USER_COT, SOFT, Acc>(a, k, mode, true, us, ux, uh, p, lam, pacc, loss, yn);
       if (!ok) {
         mode = U_FAIL;
       } else if (mode == U_RECOMP) {
@@ -1486,7 +1595,7 @@ __global__ void __launch_bounds__(256) t1_save_kernel(const RevArgs a) {
   }
 }
 
-template <class M, class Pb, class R, bool USER_COT, bool STAGES = false>
+template <class M, class Pb, class R, bool USER_COT, bool STAGES = false, bool SOFT = false>
 __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
   constexpr int D = Pb::D, NP = Pb::NP;
   constexpr int G = GroupOf<Pb>::value;
@@ -1645,13 +1754,13 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
     }
     const bool busy = (mode == U_STEP || mode == U_SIDE);
     if constexpr (STAGES) {
-      if (busy && !M::template unit_stored<Pb, R, USER_COT, Acc>(a, k, mode, true, us, yx, uh, p, sd, lam, pacc, loss))
+      if (busy && !M::template unit_stored<Pb, R, USER_COT, SOFT, Acc>(a, k, mode, true, us, yx, uh, p, sd, lam, pacc, loss))
         mode = U_FAIL;
     } else if (COLL || busy) {
       R yn[D], xin[D];
 #pragma unroll
       for (int c = 0; c < D; ++c) xin[c] = busy ? yx[c] : R(0);
-      if (!M::template unit<Pb, R, USER_COT, Acc>(a, k, mode, busy, us, xin, busy ? uh : M::IDLE_H, p, lam, pacc,
+      if (!M::template unit<Pb, R, USER_COT, SOFT, Acc>(a, k, mode, busy, us, xin, busy ? uh : M::IDLE_H, p, lam, pacc,
                                                    loss, yn) &&
           busy)
         mode = U_FAIL;
@@ -1700,6 +1809,11 @@ __global__ void __launch_bounds__(TPB_REV) reverse_k1_kernel(const RevArgs a) {
 template <class M, class Pb, class R, bool USER_COT, bool STAGES, int MINB>
 __global__ void __launch_bounds__(TPB_REV, MINB) reverse_k1_kernel_mb(const RevArgs a) {
   reverse_k1_body<M, Pb, R, USER_COT, STAGES>(a);
+}
+// The same in soft arithmetic (SoftD).
+template <class M, class Pb, bool USER_COT, bool STAGES, int MINB>
+__global__ void __launch_bounds__(TPB_REV, MINB) reverse_k1_soft_kernel(const RevArgs a) {
+  reverse_k1_body<M, Pb, double, USER_COT, STAGES, true>(a);
 }
 // The k = 1 reverse kernel of (M, Pb, R, USER_COT, STAGES), with its register cap.
 template <class M, class Pb, class R, bool USER_COT, bool STAGES = false>
@@ -1838,7 +1952,8 @@ inline bool init_step_pass(FwdArgs& a, cudaStream_t s, cudaError_t* err) {
   }
 }
 
-template <class M, class Pb, class R>
+// SOFT: the kernels in soft arithmetic (SoftD).
+template <class M, class Pb, class R, bool SOFT = false>
 inline cudaError_t fwd_dispatch(const FwdArgs& a_in, cudaStream_t s) {
   FwdArgs a = a_in;
   {
@@ -1856,6 +1971,23 @@ inline cudaError_t fwd_dispatch(const FwdArgs& a_in, cudaStream_t s) {
   }
   const long long lanes = a.n * GroupOf<Pb>::value;
   const size_t smem = (size_t)(((a.n_save + 1) & ~1) + a.segw * TPB_FWD) * sizeof(double);
+  if constexpr (SOFT) {
+    const auto launch = [&](auto c64) {
+      constexpr bool C64 = decltype(c64)::value;
+      if constexpr (stages_possible<M, Pb, R>()) {
+        if (a.stages)
+          return persistent_launch(record_soft_kernel<M, Pb, true, true, C64>, TPB_FWD, smem, lanes, s, &a);
+      }
+      if (a.stages) return cudaErrorInvalidValue;
+      if (a.y_save) return persistent_launch(record_soft_kernel<M, Pb, true, false, C64>, TPB_FWD, smem, lanes, s, &a);
+      return persistent_launch(record_soft_kernel<M, Pb, false, false, C64>, TPB_FWD, smem, lanes, s, &a);
+    };
+    if constexpr (M::kControl64) {
+      if (a.control) return launch(std::true_type{});
+    }
+    if (a.control) return cudaErrorInvalidValue;
+    return launch(std::false_type{});
+  } else {
   if (a.control) {  // FP64 step control: Tsit5 without shared weights
     if constexpr (M::kControl64 && !HasWeights<Pb>::value) {
       if constexpr (stages_possible<M, Pb, R>()) {
@@ -1877,6 +2009,7 @@ inline cudaError_t fwd_dispatch(const FwdArgs& a_in, cudaStream_t s) {
   }
   if (a.y_save) return persistent_launch(record_kernel<M, Pb, R, true, false>, TPB_FWD, smem, lanes, s, &a);
   return persistent_launch(record_kernel<M, Pb, R, false, false>, TPB_FWD, smem, lanes, s, &a);
+  }
 }
 
 #ifndef GS_T1_SAVE_PASS
@@ -1918,7 +2051,7 @@ inline bool t1_save_pass(const RevArgs& a, cudaStream_t s, cudaError_t* err) {
   }
 }
 
-template <class M, class Pb, class R>
+template <class M, class Pb, class R, bool SOFT = false>
 inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
   RevArgs a = a_in;
   a.t1_pre = 0;
@@ -1947,6 +2080,21 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
     a.t1_pre = t1_save_pass<Pb, R>(a, s, &e) ? 1 : 0;
     if (e != cudaSuccess) return e;
   }
+  if constexpr (SOFT) {
+    if constexpr (stages_possible<M, Pb, R>()) {
+      constexpr int MB = 4;  // (Lorenz 2^22: 59.6 ms at 4 CTAs per SM, 60.3 at 5)
+      if (a.stages) {
+        if (a.k != 1 || a.segw != stage_segw<M, Pb::D>()) return cudaErrorInvalidValue;
+        if (a.y_save_bar)
+          return persistent_launch(reverse_k1_soft_kernel<M, Pb, true, true, MB>, TPB_REV, smem, lanes, s, &a);
+        return persistent_launch(reverse_k1_soft_kernel<M, Pb, false, true, MB>, TPB_REV, smem, lanes, s, &a);
+      }
+    }
+    if (a.stages || a.k != 1) return cudaErrorInvalidValue;
+    if (a.y_save_bar)
+      return persistent_launch(reverse_k1_soft_kernel<M, Pb, true, false, 4>, TPB_REV, smem, lanes, s, &a);
+    return persistent_launch(reverse_k1_soft_kernel<M, Pb, false, false, 4>, TPB_REV, smem, lanes, s, &a);
+  } else {
   if constexpr (stages_possible<M, Pb, R>()) {
     if (a.stages) {
       if (a.k != 1 || a.segw != stage_segw<M, Pb::D>()) return cudaErrorInvalidValue;
@@ -1963,6 +2111,7 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
   }
   if (a.y_save_bar) return persistent_launch(reverse_kernel<M, Pb, R, true>, TPB_REV, smem, lanes, s, &a);
   return persistent_launch(reverse_kernel<M, Pb, R, false>, TPB_REV, smem, lanes, s, &a);
+  }
   }
 }
 

@@ -20,7 +20,19 @@ bool tsit5_supports(int problem, int precision) {
   return (problem == 0 || problem == 1 || problem == 4) && (precision == 0 || precision == 1);
 }
 
+// FP64 launches in soft arithmetic (SoftD, multiplications on the integer
+// pipes): every ensemble of the two-dimensional problems, and ensembles of more
+// than one warp per FP64 unit (19456 trajectories) of the three-dimensional
+// ones. Gradient of n trajectories, record + reverse, hardware against soft:
+// Lorenz 10007: 0.99 / 0.99 ms; 26000: 1.56 / 1.33; 60000: 3.07 / 2.37; 2^22:
+// 151.7 / 120.4; Van der Pol 700: 2.26 / 2.12 ms; 26000: 3.44 / 2.87; 65521: 6.83
+// / 5.01; 2^20: 73.1 / 53.5.
+bool soft_launch(int problem, int precision, int64_t n) {
+  return precision == 0 && (problem == 1 || problem == 4 || n > 608 * 32);
+}
+
 cudaError_t launch_tsit5_forward(int problem, int precision, const FwdArgs& a, cudaStream_t s) {
+  if (soft_launch(problem, precision, a.n)) return launch_tsit5_soft_forward(problem, a, s);
   switch (problem * 2 + precision) {
     case 0: return fwd_dispatch<Tsit5Method, Lorenz, double>(a, s);
     case 1: return fwd_dispatch<Tsit5Method, Lorenz, float>(a, s);
@@ -34,6 +46,7 @@ cudaError_t launch_tsit5_forward(int problem, int precision, const FwdArgs& a, c
 }
 
 cudaError_t launch_tsit5_reverse(int problem, int precision, const RevArgs& a, cudaStream_t s) {
+  if (a.k == 1 && soft_launch(problem, precision, a.n)) return launch_tsit5_soft_reverse(problem, a, s);
   switch (problem * 2 + precision) {
     case 0: return rev_dispatch<Tsit5Method, Lorenz, double>(a, s);
     case 1: return rev_dispatch<Tsit5Method, Lorenz, float>(a, s);

@@ -149,6 +149,10 @@ bool tsit5_supports(int problem, int precision);
 // gs_device.cuh); the reverse sweep for k = 1 records. Same results.
 cudaError_t launch_tsit5_soft_forward(int problem, const FwdArgs& a, cudaStream_t s);
 cudaError_t launch_tsit5_soft_reverse(int problem, const RevArgs& a, cudaStream_t s);
+// The FP64 Tsit5 kernels of Lorenz and Van der Pol with a lane per state
+// component (gs_group.cuh); the reverse sweep for k = 1 records. Same results.
+cudaError_t launch_tsit5_group_forward(int problem, const FwdArgs& a, cudaStream_t s);
+cudaError_t launch_tsit5_group_reverse(int problem, const RevArgs& a, cudaStream_t s);
 cudaError_t launch_rodas_forward(int problem, int precision, const FwdArgs& a, cudaStream_t s);
 cudaError_t launch_rodas_reverse(int problem, int precision, const RevArgs& a, cudaStream_t s);
 bool rodas_supports(int problem, int precision);

@@ -73,6 +73,14 @@ template <class Pb>
 struct LaneOf<Pb, std::void_t<typename Pb::Lane>> {
   using type = typename Pb::Lane;
 };
+template <class M, class = void>
+struct LaneMethodOf {
+  using type = M;
+};
+template <class M>
+struct LaneMethodOf<M, std::void_t<typename M::LaneMethod>> {
+  using type = typename M::LaneMethod;
+};
 template <class Pb>
 __device__ __forceinline__ bool group_leader() {
   return (threadIdx.x & (GroupOf<Pb>::value - 1)) == 0;
@@ -895,6 +903,8 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
   static_assert(!STAGES || (SAVES && M::kStages), "stored stages need side steps and a method that exposes stages");
   constexpr int D = Pb::D, NP = Pb::NP;
   using Carry = typename M::template Carry<Pb, R>;
+  // the per-lane problem of the starting step; a network in lane groups stays in its group form
+  using LanePb = typename std::conditional<HasWeights<Pb>::value, Pb, typename LaneOf<Pb>::type>::type;
   static_assert(!SOFT || (M::kSoft && std::is_same<R, double>::value), "soft arithmetic is FP64's");
   extern __shared__ double smem[];
   const int ns = a.n_save;
@@ -973,10 +983,10 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
               h = a.y_final[k];  // the starting-step pass's result (this slot is rewritten when k ends)
             } else if constexpr (C64) {
               double fd[D];
-              Pb::f(yd, pd, fd);
-              h = initial_step_f64<Pb, M::ORDER>(yd, pd, fd, a.t0, t1, a.rtol, a.atol);
+              LanePb::f(yd, pd, fd);
+              h = initial_step_f64<LanePb, M::ORDER>(yd, pd, fd, a.t0, t1, a.rtol, a.atol);
             } else {
-              h = initial_step_f32<Pb, M::ORDER>(yf, pf, ff, a.t0, t1, a.rtol, a.atol);
+              h = initial_step_f32<LanePb, M::ORDER>(yf, pf, ff, a.t0, t1, a.rtol, a.atol);
             }
           }
           fin = fin && positive(h) && finite_nonneg(h);
@@ -1067,7 +1077,8 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
         // overwritten by the next trial if this one is rejected), so that they
         // are not held in registers across the step-size decision
         if (hard) solved = M::template trial_s<Pb, R>(xin, pin, hx, cin, yn, e, next, sd);
-        if (is_side) {
+        if (is_side && !group_leader<Pb>()) {
+        } else if (is_side) {
           constexpr int SP = M::template side_payload<D>();
           if constexpr (side_blocks<SP>()) {  // this trajectory's block, 16-byte vector stores
             double* dst = a.side_stg + ((long long)k * ns + jp) * SP;
@@ -1319,11 +1330,15 @@ __device__ __forceinline__ void write_nan(const RevArgs& a, long long k) {
 
 template <int NP, int D, class R, class Acc>
 __device__ __forceinline__ void write_grad(const RevArgs& a, long long k, const Acc& pacc, const R (&lam)[D],
-                                           double loss) {
+                                           double loss, bool leader = true) {
   const long long n = a.n;
+  double pb[NP];  // (a group's lanes read one another's sums)
+#pragma unroll
+  for (int q = 0; q < NP; ++q) pb[q] = pacc.get(q);
+  if (!leader) return;
   if (a.params_bar)
 #pragma unroll
-    for (int q = 0; q < NP; ++q) a.params_bar[q * n + k] = pacc.get(q);
+    for (int q = 0; q < NP; ++q) a.params_bar[q * n + k] = pb[q];
   if (a.y0_bar)
 #pragma unroll
     for (int c = 0; c < D; ++c) a.y0_bar[c * n + k] = (double)lam[c];
@@ -1386,8 +1401,15 @@ template <>
 struct WeightAcc<NeuralRobertsonGroup> {
   using type = NrGroupAcc;
 };
+// Lane-per-component problems (gs_group.cuh) bring theirs.
+template <class Pb>
+struct GroupAccOf {
+  using type = void;
+};
 template <class Pb, class R>
-using AccFor = typename std::conditional<HasWeights<Pb>::value, typename WeightAcc<Pb>::type, AccOf<R, Pb::NP>>::type;
+using AccFor = typename std::conditional<
+    HasWeights<Pb>::value, typename WeightAcc<Pb>::type,
+    typename std::conditional<(GroupOf<Pb>::value > 1), typename GroupAccOf<Pb>::type, AccOf<R, Pb::NP>>::type>::type;
 // Dynamic shared memory a shared-weight accumulator stages its factors in.
 template <class Pb>
 constexpr size_t weight_stage_bytes() {
@@ -1635,7 +1657,7 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
         got = need ? stat_next : -1;
         if (need) stat_next += stat_stride;
       } else {
-        got = warp_ticket(a.work, need);
+        got = from_leader<Pb>(warp_ticket(a.work, need && group_leader<Pb>()));
       }
       if (need) {
         if (got < n) {
@@ -1770,7 +1792,7 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
       k = -1;
     }
     if (mode == U_DONE) {
-      if (group_leader<Pb>()) write_grad<NP, D, R>(a, k, pacc, lam, loss);
+      write_grad<NP, D, R>(a, k, pacc, lam, loss, group_leader<Pb>());
       k = -1;
     }
   }
@@ -1961,11 +1983,11 @@ inline cudaError_t fwd_dispatch(const FwdArgs& a_in, cudaStream_t s) {
     a.h0_pre = 0;
     if constexpr (M::kControl64 && !HasWeights<Pb>::value) {  // (FP64 control: no shared weights)
       if (a.control)
-        init_step_pass<M, typename LaneOf<Pb>::type, R, true>(a, s, &e);
+        init_step_pass<typename LaneMethodOf<M>::type, typename LaneOf<Pb>::type, R, true>(a, s, &e);
       else
-        init_step_pass<M, typename LaneOf<Pb>::type, R, false>(a, s, &e);
+        init_step_pass<typename LaneMethodOf<M>::type, typename LaneOf<Pb>::type, R, false>(a, s, &e);
     } else {
-      init_step_pass<M, typename LaneOf<Pb>::type, R, false>(a, s, &e);
+      init_step_pass<typename LaneMethodOf<M>::type, typename LaneOf<Pb>::type, R, false>(a, s, &e);
     }
     if (e != cudaSuccess) return e;
   }
@@ -2109,8 +2131,12 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
     if (a.y_save_bar) return persistent_launch(reverse_k1_entry<M, Pb, R, true>(), TPB_REV, smem, lanes, s, &a);
     return persistent_launch(reverse_k1_entry<M, Pb, R, false>(), TPB_REV, smem, lanes, s, &a);
   }
-  if (a.y_save_bar) return persistent_launch(reverse_kernel<M, Pb, R, true>, TPB_REV, smem, lanes, s, &a);
-  return persistent_launch(reverse_kernel<M, Pb, R, false>, TPB_REV, smem, lanes, s, &a);
+  if constexpr (GroupOf<Pb>::value > 1) {
+    return cudaErrorInvalidValue;  // (lane groups sweep k = 1 records)
+  } else {
+    if (a.y_save_bar) return persistent_launch(reverse_kernel<M, Pb, R, true>, TPB_REV, smem, lanes, s, &a);
+    return persistent_launch(reverse_kernel<M, Pb, R, false>, TPB_REV, smem, lanes, s, &a);
+  }
   }
   }
 }

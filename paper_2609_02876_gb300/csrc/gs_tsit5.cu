@@ -20,7 +20,7 @@ bool tsit5_supports(int problem, int precision) {
   return (problem == 0 || problem == 1 || problem == 4) && (precision == 0 || precision == 1);
 }
 
-// FP64 launches in soft arithmetic (SoftD, multiplications on the integer
+// Other FP64 launches in soft arithmetic (SoftD, multiplications on the integer
 // pipes): every ensemble of the two-dimensional problems, and ensembles of more
 // than one warp per FP64 unit (19456 trajectories) of the three-dimensional
 // ones. Gradient of n trajectories, record + reverse, hardware against soft:
@@ -31,7 +31,17 @@ bool soft_launch(int problem, int precision, int64_t n) {
   return precision == 0 && (problem == 1 || problem == 4 || n > 608 * 32);
 }
 
+// FP64 launches with a lane per state component (gs_group.cuh): Lorenz and Van
+// der Pol up to 9728 trajectories (Lorenz: two group warps per FP64 unit; Van der
+// Pol: one). Gradient, record + reverse, per-lane against groups: Lorenz 1024:
+// 0.96 / 0.64 ms; 9728: 0.99 / 0.85; 10007: 0.99 / 1.15 (some units hold three);
+// Van der Pol 700: 2.12 / 1.95; 9728: 2.24 / 2.04; 14000: 2.26 / 2.64.
+bool group_launch(int problem, int precision, int64_t n) {
+  return precision == 0 && (problem == 0 || problem == 1) && n <= 9728;
+}
+
 cudaError_t launch_tsit5_forward(int problem, int precision, const FwdArgs& a, cudaStream_t s) {
+  if (group_launch(problem, precision, a.n)) return launch_tsit5_group_forward(problem, a, s);
   if (soft_launch(problem, precision, a.n)) return launch_tsit5_soft_forward(problem, a, s);
   switch (problem * 2 + precision) {
     case 0: return fwd_dispatch<Tsit5Method, Lorenz, double>(a, s);
@@ -46,6 +56,7 @@ cudaError_t launch_tsit5_forward(int problem, int precision, const FwdArgs& a, c
 }
 
 cudaError_t launch_tsit5_reverse(int problem, int precision, const RevArgs& a, cudaStream_t s) {
+  if (a.k == 1 && group_launch(problem, precision, a.n)) return launch_tsit5_group_reverse(problem, a, s);
   if (a.k == 1 && soft_launch(problem, precision, a.n)) return launch_tsit5_soft_reverse(problem, a, s);
   switch (problem * 2 + precision) {
     case 0: return rev_dispatch<Tsit5Method, Lorenz, double>(a, s);

@@ -1,7 +1,8 @@
 """The integer FP64 multiplication of the Tsit5 kernels (SoftD): bit for bit the
 IEEE product on the CPU (where the compiler's multiplication is the reference),
 its range test, and on the GPU the same results from ensembles that take it and
-ones that do not, with values in and out of its range."""
+ones that do not, with values in and out of its range; and the lane-per-component
+form of small ensembles against the per-lane forms."""
 import os
 import subprocess
 
@@ -77,12 +78,14 @@ def _grad(problem, p, y, wl, **kw):
 @pytest.mark.gpu
 @pytest.mark.parametrize("control", ["fast", "fp64"])
 @pytest.mark.parametrize("extreme", [False, True])
-def test_lorenz_same_bits_on_both_sides_of_the_line(extreme, control):
-    """19457 trajectories take the integer products, their first 700 alone do
-    not: same bits, with trajectories on the z axis (zero states and slopes),
-    at the origin, of tiny and of huge states, and with zero parameters."""
+@pytest.mark.parametrize("n", [9729, 19457])
+def test_lorenz_same_bits_on_both_sides_of_the_lines(n, extreme, control):
+    """19457 trajectories take the integer products, 9729 the hardware ones, and
+    the first 700 alone a lane per component: same bits, with trajectories on the
+    z axis (zero states and slopes), at the origin, of tiny and of huge states,
+    and with zero parameters."""
     B.build()
-    n, m = 19457, 700
+    m = 700
     wl = W.make("lorenz", n)
     p, y = wl["params"].copy(), wl["y0"].copy()
     if extreme:
@@ -112,6 +115,33 @@ def test_lorenz_same_bits_on_both_sides_of_the_line(extreme, control):
     f1 = api.solve("lorenz", P, Y, *args, **kw)
     f2 = api.solve("lorenz", P[:, :m].contiguous(), Y[:, :m].contiguous(), *args, **kw)
     assert torch.equal(f1["y_final"][:, :m][:, ok], f2["y_final"][:, ok])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("problem", ["lorenz", "vdp"])
+@pytest.mark.parametrize("m", [1, 9, 31, 9728])
+def test_lane_per_component_ragged_sizes(problem, m):
+    """Up to 9728 trajectories run a lane per component, 9729 a lane each: same
+    bits for ragged last groups and warps, user cotangents included."""
+    B.build()
+    wl = W.make(problem, 9729)
+    P, Y = dev(wl["params"].T), dev(wl["y0"].T)
+    args = (wl["t0"], wl["t1"], wl["save_t"], wl["rtol"], wl["atol"])
+    Ps, Ys = P[:, :m].contiguous(), Y[:, :m].contiguous()
+    a = api.solve_grad(problem, P, Y, *args, layout="soa")
+    b = api.solve_grad(problem, Ps, Ys, *args, layout="soa")
+    for k in ("loss", "params_bar", "y0_bar"):
+        assert torch.equal(a[k][..., :m], b[k]), k
+    cot = torch.randn((len(wl["save_t"]), Y.shape[0], 9729), dtype=torch.float64, device="cuda",
+                      generator=torch.Generator("cuda").manual_seed(1))
+    for stages in (False, True):
+        ra, ya, _ = api.forward_record(problem, P, Y, *args, layout="soa", record_stages=stages, ckpt_k=1)
+        rb, yb, _ = api.forward_record(problem, Ps, Ys, *args, layout="soa", record_stages=stages, ckpt_k=1)
+        assert torch.equal(ya[..., :m], yb)
+        ga = api.reverse(ra, P, Y, cot, layout="soa")
+        gb = api.reverse(rb, Ps, Ys, cot[..., :m].contiguous(), layout="soa")
+        for k in ("params_bar", "y0_bar"):
+            assert torch.equal(ga[k][:, :m], gb[k]), k
 
 
 @pytest.mark.gpu

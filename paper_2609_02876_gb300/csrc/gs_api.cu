@@ -100,7 +100,19 @@ struct Counters {
 
 }  // namespace
 
+// What decides the sizes of a record's buffers (besides the device).
+struct RecordKey {
+  int problem, method, precision, k, stages, n_save;
+  int64_t n;
+  double rtol;
+  bool operator==(const RecordKey& o) const {
+    return problem == o.problem && method == o.method && precision == o.precision && k == o.k && stages == o.stages &&
+           n_save == o.n_save && n == o.n && rtol == o.rtol;
+  }
+};
+
 struct gs_record {
+  RecordKey key = {};
   int device = 0;
   int problem = 0, method = GS_METHOD_TSIT5, precision = GS_FP64;
   int d = 0, P = 0, k = 0, segw = 0;
@@ -152,6 +164,20 @@ gs_status cuda_fail(cudaError_t e) {
   return GS_ERR_CUDA;
 }
 
+bool pool_drain();
+
+// cudaMalloc; if it fails, once more after the pool of freed records has given
+// its memory back.
+template <class T>
+cudaError_t dev_alloc(T** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    if (pool_drain()) e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+
 void free_arrays(gs_record* r) {
   cudaFree(r->head);
   cudaFree(r->S);
@@ -180,11 +206,11 @@ gs_status ensure_arrays(gs_record* r, int64_t n, int d) {
   const int64_t m = n > 0 ? n : 1;
   d = kMaxDim;  // y(t1) sized for any problem, so a reused workspace never reallocates for d
   cudaError_t e;
-  if ((e = cudaMalloc(&r->head, m * sizeof(long long))) != cudaSuccess) return cuda_fail(e);
-  if ((e = cudaMalloc(&r->S, m * sizeof(int32_t))) != cudaSuccess) return cuda_fail(e);
-  if ((e = cudaMalloc(&r->natt, m * sizeof(int32_t))) != cudaSuccess) return cuda_fail(e);
-  if ((e = cudaMalloc(&r->status, m * sizeof(int32_t))) != cudaSuccess) return cuda_fail(e);
-  if ((e = cudaMalloc(&r->y_final, m * d * sizeof(double))) != cudaSuccess) return cuda_fail(e);
+  if ((e = dev_alloc(&r->head, m * sizeof(long long))) != cudaSuccess) return cuda_fail(e);
+  if ((e = dev_alloc(&r->S, m * sizeof(int32_t))) != cudaSuccess) return cuda_fail(e);
+  if ((e = dev_alloc(&r->natt, m * sizeof(int32_t))) != cudaSuccess) return cuda_fail(e);
+  if ((e = dev_alloc(&r->status, m * sizeof(int32_t))) != cudaSuccess) return cuda_fail(e);
+  if ((e = dev_alloc(&r->y_final, m * d * sizeof(double))) != cudaSuccess) return cuda_fail(e);
   r->n_cap = m;
   return GS_OK;
 }
@@ -194,7 +220,7 @@ gs_status ensure_arena(gs_record* r, long long segs, int segw) {
   cudaFree(r->arena);
   r->arena = nullptr;
   r->arena_cap = 0;
-  cudaError_t e = cudaMalloc(&r->arena, (size_t)segs * segw * sizeof(double));
+  cudaError_t e = dev_alloc(&r->arena, (size_t)segs * segw * sizeof(double));
   if (e != cudaSuccess) return cuda_fail(e);
   r->arena_cap = segs;
   return GS_OK;
@@ -202,7 +228,7 @@ gs_status ensure_arena(gs_record* r, long long segs, int segw) {
 
 gs_status ensure_counters(gs_record* r) {
   if (r->ctr) return GS_OK;
-  cudaError_t e = cudaMalloc(&r->ctr, sizeof(Counters));
+  cudaError_t e = dev_alloc(&r->ctr, sizeof(Counters));
   if (e != cudaSuccess) return cuda_fail(e);
   e = cudaMallocHost(&r->ctr_host, sizeof(Counters));
   if (e != cudaSuccess) return cuda_fail(e);
@@ -229,6 +255,66 @@ void destroy(gs_record* r) {
   cudaFree(r->wpart);
   cudaFreeHost(r->ctr_host);
   delete r;
+}
+
+// Freed records of at most POOL_RECORD_BYTES, kept for the next
+// gs_forward_record of the same call signature (a training loop records and
+// frees one per step; allocating and freeing its buffers took 0.45 ms of a 2.0 ms
+// step at 10007 Lorenz trajectories). At most POOL_RECORDS of them; the oldest is
+// released for a newer one, and all of them when an allocation fails. A record
+// enters the pool after the device has finished all work, as cudaFree would have
+// waited for, so any stream may use it next.
+constexpr size_t POOL_RECORD_BYTES = size_t(128) << 20;
+constexpr size_t POOL_RECORDS = 2;
+std::mutex g_pool_mu;
+std::vector<gs_record*> g_pool;  // oldest first
+
+gs_record* pool_take(const RecordKey& key) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  for (size_t i = 0; i < g_pool.size(); ++i) {
+    gs_record* r = g_pool[i];
+    if (r->device == dev && r->key == key) {
+      g_pool.erase(g_pool.begin() + i);
+      return r;
+    }
+  }
+  return nullptr;
+}
+
+bool pool_put(gs_record* r) {  // false: the caller releases it
+  if (!r || !r->arena || record_bytes(r) > POOL_RECORD_BYTES) return false;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev != r->device) return false;
+  if (cudaDeviceSynchronize() != cudaSuccess) return false;
+  cudaFree(r->fwd_base);
+  cudaFree(r->fwd_seg);
+  r->fwd_base = r->fwd_seg = nullptr;
+  gs_record* old = nullptr;
+  try {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (g_pool.size() >= POOL_RECORDS) {
+      old = g_pool.front();
+      g_pool.erase(g_pool.begin());
+    }
+    g_pool.push_back(r);
+  } catch (...) {
+    destroy(old);
+    return false;
+  }
+  destroy(old);
+  return true;
+}
+
+bool pool_drain() {  // whether anything was released
+  std::vector<gs_record*> all;
+  {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    all.swap(g_pool);
+  }
+  for (gs_record* r : all) destroy(r);
+  return !all.empty();
 }
 
 struct Call {
@@ -322,9 +408,9 @@ gs_status check_common(int problem_id, int64_t n, const double* params, const do
   return GS_OK;
 }
 
-// Runs the record kernel into r, growing the arena until it fits.
-gs_status run_record(gs_record* r, const Call& c, int64_t n, const double* params, const double* y0,
-                     const float* shared_w, double* y_save, cudaStream_t s) {
+// Enqueues the record kernel into r (counters zeroed first, statuses to `status`).
+gs_status enqueue_record(gs_record* r, const Call& c, int64_t n, const double* params, const double* y0,
+                         const float* shared_w, double* y_save, int32_t* status, cudaStream_t s) {
   FwdArgs a;
   std::memset(&a, 0, sizeof(a));
   a.n = n;
@@ -342,52 +428,73 @@ gs_status run_record(gs_record* r, const Call& c, int64_t n, const double* param
   std::memcpy(a.save_t, r->save_t, sizeof(double) * r->n_save);
   a.y_save = y_save;
   a.step_counts = c.step_counts;
+  a.k = r->k;
+  a.segw = r->segw;
+  a.arena_block = r->arena_block;
+  a.stages = r->stages;
+  a.side_stg = r->stages ? r->side_stg : nullptr;
+  cudaError_t e = cudaMemsetAsync(r->ctr, 0, sizeof(Counters), s);
+  if (e != cudaSuccess) return cuda_fail(e);
+  a.arena = r->arena;
+  a.arena_cap = r->arena_cap;
+  a.arena_top = &r->ctr->arena_top;
+  a.overflow = &r->ctr->overflow;
+  a.any_failed = &r->ctr->any_failed;
+  a.head = r->head;
+  a.S = r->S;
+  a.natt = r->natt;
+  a.status = status;
+  a.y_final = r->y_final;
+  a.work = &r->ctr->work_fwd;
+  if (c.kernel_ms) cudaEventRecord(r->ev[0], s);
+  e = launch_forward_m(c.method, c.problem, c.precision, a, s);
+  if (e != cudaSuccess) return GS_ERR_CUDA;
+  if (c.kernel_ms) cudaEventRecord(r->ev[1], s);
+  return GS_OK;
+}
+
+// Brings the counters to the host and waits for the work queued on s.
+gs_status wait_counters(gs_record* r, const Call& c, cudaStream_t s) {
+  const cudaError_t e = cudaMemcpyAsync(r->ctr_host, r->ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s);
+  if (e != cudaSuccess) return GS_ERR_CUDA;
+  return wait_stream(s, c.timeout_ms);
+}
+
+// After a record whose arena was large enough.
+void record_done(gs_record* r, const Call& c) {
+  if (c.kernel_ms) cudaEventElapsedTime(&c.kernel_ms[0], r->ev[0], r->ev[1]);
+  if (c.record_info) {
+    c.record_info[0] = r->k;
+    c.record_info[1] = r->stages;
+  }
+  r->nseg_total = (long long)r->ctr_host->arena_top;
+}
+
+// The arena was too small: size it to the demand just measured (+1/8), as a
+// compact record if the stored-stage one does not fit.
+gs_status grow_arena(gs_record* r) {
+  const long long need = (long long)r->ctr_host->arena_top;
+  gs_status st = ensure_arena(r, need + need / 8 + 1024, r->segw);
+  if (st == GS_ERR_OOM && r->stages) {
+    r->stages = 0;
+    r->segw = segw_of(r->d, r->k);
+    st = ensure_arena(r, need + need / 8 + 1024, r->segw);
+  }
+  return st;
+}
+
+// Runs the record kernel into r, growing the arena until it fits.
+gs_status run_record(gs_record* r, const Call& c, int64_t n, const double* params, const double* y0,
+                     const float* shared_w, double* y_save, int32_t* status, cudaStream_t s) {
   for (int attempt = 0; attempt < 3; ++attempt) {
-    a.k = r->k;
-    a.segw = r->segw;
-    a.arena_block = r->arena_block;
-    a.stages = r->stages;
-    a.side_stg = r->stages ? r->side_stg : nullptr;
-    cudaError_t e = cudaMemsetAsync(r->ctr, 0, sizeof(Counters), s);
-    if (e != cudaSuccess) return cuda_fail(e);
-    a.arena = r->arena;
-    a.arena_cap = r->arena_cap;
-    a.arena_top = &r->ctr->arena_top;
-    a.overflow = &r->ctr->overflow;
-    a.any_failed = &r->ctr->any_failed;
-    a.head = r->head;
-    a.S = r->S;
-    a.natt = r->natt;
-    a.status = r->status;
-    a.y_final = r->y_final;
-    a.work = &r->ctr->work_fwd;
-    if (c.kernel_ms) cudaEventRecord(r->ev[0], s);
-    e = launch_forward_m(c.method, c.problem, c.precision, a, s);
-    if (e != cudaSuccess) return GS_ERR_CUDA;
-    if (c.kernel_ms) cudaEventRecord(r->ev[1], s);
-    e = cudaMemcpyAsync(r->ctr_host, r->ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s);
-    if (e != cudaSuccess) return GS_ERR_CUDA;
-    const gs_status ws = wait_stream(s, c.timeout_ms);
-    if (ws != GS_OK) return ws;
+    gs_status st = enqueue_record(r, c, n, params, y0, shared_w, y_save, status, s);
+    if (st == GS_OK) st = wait_counters(r, c, s);
+    if (st != GS_OK) return st;
     if (!r->ctr_host->overflow) {
-      if (c.kernel_ms) cudaEventElapsedTime(&c.kernel_ms[0], r->ev[0], r->ev[1]);
-      if (c.record_info) {
-        c.record_info[0] = r->k;
-        c.record_info[1] = r->stages;
-      }
-      r->nseg_total = (long long)r->ctr_host->arena_top;
+      record_done(r, c);
       return GS_OK;
     }
-    // The arena was too small: size it to the demand just measured (+1/8) and rerun
-    // (as a compact record if the stored-stage one does not fit).
-    const long long need = (long long)r->ctr_host->arena_top;
-    gs_status st = ensure_arena(r, need + need / 8 + 1024, r->segw);
-    if (st == GS_ERR_OOM && r->stages) {
-      r->stages = 0;
-      r->segw = segw_of(r->d, r->k);
-      st = ensure_arena(r, need + need / 8 + 1024, r->segw);
-    }
-    if (st != GS_OK) return st;
+    if ((st = grow_arena(r)) != GS_OK) return st;
   }
   return GS_ERR_OOM;
 }
@@ -397,12 +504,24 @@ gs_status run_record(gs_record* r, const Call& c, int64_t n, const double* param
 // expected record takes at most half of the free device memory, else a
 // 128-byte segment of 14 - d steps (one checkpoint per 14 - d steps).
 int auto_ckpt_k(const gs_record* r, int problem, int d, int64_t n) {
+  if (r->arena && r->segw == segw_of(d, 1) && r->arena_cap >= (n > 0 ? n : 1) * (long long)(step_guess(problem) + 1))
+    return 1;  // held from an earlier call of this size
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = 0;
   const size_t held = (size_t)r->arena_cap * r->segw * sizeof(double);  // reusable by this record
   const double want = 1.25 * (double)(n > 0 ? n : 1) * step_guess(problem) * segw_of(d, 1) * sizeof(double);
   if (want <= 0.5 * (double)(free_b + held)) return 1;
   return 14 - d > 1 ? 14 - d : 1;
+}
+
+// Whether r already holds a stored-stage record for this ensemble (a workspace
+// used again): nothing would be allocated, so the free memory, which takes a
+// driver call to learn, does not matter.
+bool holds_stages(const gs_record* r, const Call& c, int64_t n, int n_save, double rtol) {
+  const long long m = n > 0 ? n : 1;
+  return r->arena && r->segw == stage_segw_of(c.method, c.pi.d) &&
+         r->arena_cap >= m * (step_guess(c.problem, rtol, c.method) + 1) &&
+         r->side_cap >= (size_t)m * (size_t)(n_save > 0 ? n_save : 1) * (size_t)stage_side_payload(c.method, c.pi.d);
 }
 
 // Stored stages when the caller allows them (gs_solve_grad), the method and
@@ -416,6 +535,7 @@ bool choose_stages(const gs_record* r, const Call& c, int64_t n, int n_save, dou
     return false;
   if (c.precision != GS_FP64 || c.pi.n_shared > 0 || c.k > 1) return false;
   if (stage_segw_of(c.method, c.pi.d) > MAX_STAGE_SEGW) return false;
+  if (holds_stages(r, c, n, n_save, rtol)) return true;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
   const double held = (double)r->arena_cap * r->segw * sizeof(double) + (double)r->side_cap * sizeof(double);
@@ -437,7 +557,7 @@ gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double
   r->stages = (allow_stages && choose_stages(r, c, n, n_save, rtol)) ? 1 : 0;
   r->k = r->stages ? 1 : (c.k > 0 ? c.k : (c.pi.n_shared > 0 ? 1 : auto_ckpt_k(r, c.problem, c.pi.d, n)));
   if (c.pi.n_shared > 0 && !r->wpart) {
-    const cudaError_t e = cudaMalloc(&r->wpart, (size_t)ude_max_warps() * WPART_BYTES_PER_WARP);
+    const cudaError_t e = dev_alloc(&r->wpart, (size_t)ude_max_warps() * WPART_BYTES_PER_WARP);
     if (e != cudaSuccess) return cuda_fail(e);
   }
   r->n = n;
@@ -459,7 +579,7 @@ gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double
       cudaFree(r->side_stg);
       r->side_stg = nullptr;
       r->side_cap = 0;
-      const cudaError_t e = cudaMalloc(&r->side_stg, need * sizeof(double));
+      const cudaError_t e = dev_alloc(&r->side_stg, need * sizeof(double));
       if (e != cudaSuccess) {
         r->stages = 0;  // fall back to the compact record
         r->k = c.k > 0 ? c.k : auto_ckpt_k(r, c.problem, c.pi.d, n);
@@ -507,7 +627,7 @@ gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double
 
 gs_status launch_reverse(const gs_record* r, const double* params, const float* shared_w,
                          const double* y_save_bar, double* loss, double* params_bar, double* y0_bar,
-                         float* shared_w_bar, cudaStream_t s) {
+                         float* shared_w_bar, const int32_t* status, bool fresh_counters, cudaStream_t s) {
   RevArgs a;
   std::memset(&a, 0, sizeof(a));
   a.n = r->n;
@@ -522,7 +642,7 @@ gs_status launch_reverse(const gs_record* r, const double* params, const float* 
   a.loss = loss;
   a.params_bar = params_bar;
   a.y0_bar = y0_bar;
-  a.status = r->status;
+  a.status = status;
   a.arena = r->arena;
   a.arena_cap = r->arena_cap;
   a.head = r->head;
@@ -535,7 +655,7 @@ gs_status launch_reverse(const gs_record* r, const double* params, const float* 
   a.stages = r->stages;
   a.side_stg = r->stages ? r->side_stg : nullptr;
   a.tc_error = &r->ctr->tc_error;
-  cudaError_t e = cudaMemsetAsync(&r->ctr->work_rev, 0, sizeof(unsigned long long), s);
+  cudaError_t e = fresh_counters ? cudaSuccess : cudaMemsetAsync(&r->ctr->work_rev, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return GS_ERR_CUDA;
   e = launch_reverse_m(r->method, r->problem, r->precision, a, s);
   return e == cudaSuccess ? GS_OK : GS_ERR_CUDA;
@@ -575,8 +695,8 @@ gs_status ensure_fwd_index(const gs_record* r, cudaStream_t s) {
   if (r->fwd_base) return GS_OK;
   long long* base = nullptr;
   long long* seg = nullptr;
-  cudaError_t e = cudaMalloc(&base, (size_t)r->n * sizeof(long long));
-  if (e == cudaSuccess) e = cudaMalloc(&seg, (size_t)(r->nseg_total > 0 ? r->nseg_total : 1) * sizeof(long long));
+  cudaError_t e = dev_alloc(&base, (size_t)r->n * sizeof(long long));
+  if (e == cudaSuccess) e = dev_alloc(&seg, (size_t)(r->nseg_total > 0 ? r->nseg_total : 1) * sizeof(long long));
   if (e == cudaSuccess) e = cudaMemsetAsync(&r->ctr->work_jvp, 0, sizeof(unsigned long long), s);
   if (e == cudaSuccess)
     e = launch_fwd_index(r->n, r->head, r->S, r->status, r->arena, r->arena_cap, r->k, r->segw, &r->ctr->work_jvp,
@@ -620,25 +740,49 @@ gs_status jvp_common(const gs_record* r, const double* params, const double* y0,
   return GS_OK;
 }
 
-// Record then reverse into workspace r (the body of gs_solve_grad[_ctx]).
+bool overlap(const void* x, size_t xb, const void* y, size_t yb) {
+  const char *p = static_cast<const char*>(x), *q = static_cast<const char*>(y);
+  return p && q && p < q + yb && q < p + xb;
+}
+
+// Record then reverse into workspace r (the body of gs_solve_grad[_ctx]). The
+// reverse sweep is queued right behind the record, and the host waits once, for
+// both: if the arena turned out too small, the sweep has met segment indices past
+// its end (which it turns into NaN gradients), and both run again on the grown
+// arena. Only calls whose outputs overlap their inputs, or with a wait deadline,
+// wait for the record first. At 1024 Lorenz trajectories the round trip between
+// the two, the status copy and the memory query were 70 us of an 831 us call.
 gs_status solve_grad_in(gs_record* r, const Call& c, int64_t n, const double* params, const double* y0,
                         const float* shared_w, double t0, double t1, const double* save_t, int n_save, double rtol,
                         double atol, cudaStream_t s, double* loss_out, double* params_bar, double* y0_bar,
                         float* shared_w_bar, int32_t* traj_status, bool allow_stages) {
   gs_status st = setup_record(r, c, n, t0, t1, save_t, n_save, rtol, atol, allow_stages);
   if (st != GS_OK) return st;
-  st = run_record(r, c, n, params, y0, shared_w, nullptr, s);
-  if (st != GS_OK) return st;
-  if (c.kernel_ms) cudaEventRecord(r->ev[2], s);
-  st = launch_reverse(r, params, shared_w, nullptr, loss_out, params_bar, y0_bar, shared_w_bar, s);
-  if (st != GS_OK) return st;
-  if (c.kernel_ms) cudaEventRecord(r->ev[3], s);
-  cudaError_t e = cudaMemcpyAsync(traj_status, r->status, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
-  if (e != cudaSuccess) return GS_ERR_CUDA;
-  e = cudaMemcpyAsync(&r->ctr_host->tc_error, &r->ctr->tc_error, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e != cudaSuccess) return GS_ERR_CUDA;
-  st = wait_stream(s, c.timeout_ms);
-  if (st != GS_OK) return st;
+  const size_t nb = (size_t)n * sizeof(double);
+  const void* outs[5] = {loss_out, params_bar, y0_bar, shared_w_bar, traj_status};
+  const size_t outb[5] = {nb, nb * c.pi.P, nb * c.pi.d, sizeof(float) * c.pi.n_shared, sizeof(int32_t) * (size_t)n};
+  const void* ins[3] = {params, y0, shared_w};
+  const size_t inb[3] = {nb * c.pi.P, nb * c.pi.d, sizeof(float) * c.pi.n_shared};
+  bool apart = c.timeout_ms > 0.0;
+  for (int i = 0; i < 5; ++i)
+    for (int j = 0; j < 3; ++j) apart = apart || overlap(outs[i], outb[i], ins[j], inb[j]);
+  int32_t* status = apart ? r->status : traj_status;
+  if (apart && (st = run_record(r, c, n, params, y0, shared_w, nullptr, status, s)) != GS_OK) return st;
+  for (int attempt = 0;; ++attempt) {
+    if (attempt == 3) return GS_ERR_OOM;
+    if (!apart && (st = enqueue_record(r, c, n, params, y0, shared_w, nullptr, status, s)) != GS_OK) return st;
+    if (c.kernel_ms) cudaEventRecord(r->ev[2], s);
+    st = launch_reverse(r, params, shared_w, nullptr, loss_out, params_bar, y0_bar, shared_w_bar, status, true, s);
+    if (st != GS_OK) return st;
+    if (c.kernel_ms) cudaEventRecord(r->ev[3], s);
+    if (apart && cudaMemcpyAsync(traj_status, r->status, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s) !=
+                     cudaSuccess)
+      return GS_ERR_CUDA;
+    if ((st = wait_counters(r, c, s)) != GS_OK) return st;
+    if (!r->ctr_host->overflow) break;
+    if ((st = grow_arena(r)) != GS_OK) return st;
+  }
+  record_done(r, c);
   if (c.kernel_ms) cudaEventElapsedTime(&c.kernel_ms[1], r->ev[2], r->ev[3]);
   if (r->ctr_host->tc_error) return GS_ERR_CUDA;
   return r->ctr_host->any_failed ? GS_ERR_TRAJ_FAILED : GS_OK;
@@ -682,7 +826,7 @@ gs_status solve_grad_chunked(gs_record* r, const Call& c, int64_t n, int64_t ch,
     cudaFree(r->chunk_buf);
     r->chunk_buf = nullptr;
     r->chunk_cap = 0;
-    if (cudaMalloc(&r->chunk_buf, need * sizeof(double)) != cudaSuccess) {
+    if (dev_alloc(&r->chunk_buf, need * sizeof(double)) != cudaSuccess) {
       cudaGetLastError();  // no staging: the one-piece call
       return solve_grad_in(r, c, n, params, y0, nullptr, t0, t1, save_t, n_save, rtol, atol, s, loss_out,
                            params_bar, y0_bar, nullptr, traj_status, allow_stages);
@@ -776,7 +920,7 @@ gs_status host_pipe(int dev, size_t in_bytes, size_t out_bytes, HostPipe** out) 
     }
     hp->in_bytes = hp->out_bytes = 0;
     for (int i = 0; i < 2; ++i)
-      if (cudaMalloc(&hp->in[i], in_bytes) != cudaSuccess || cudaMalloc(&hp->out[i], out_bytes) != cudaSuccess) {
+      if (dev_alloc(&hp->in[i], in_bytes) != cudaSuccess || dev_alloc(&hp->out[i], out_bytes) != cudaSuccess) {
         cudaGetLastError();
         return GS_ERR_OOM;
       }
@@ -841,13 +985,16 @@ gs_status gs_forward_record(int problem_id, int64_t n, const double* params, con
   if (st != GS_OK) return st;
   if (n > 0 && !traj_status) return GS_ERR_INVALID_ARG;
   c.timeout_ms = 0.0;  // the record handle owns the work: wait for it
-  gs_record* r = new (std::nothrow) gs_record();
+  const RecordKey key = {c.problem, c.method, c.precision, c.k, c.record_stages, n_save, n, rtol};
+  gs_record* r = pool_take(key);
+  if (!r) r = new (std::nothrow) gs_record();
   if (!r) return GS_ERR_OOM;
+  r->key = key;
   st = setup_record(r, c, n, t0, t1, save_t, n_save, rtol, atol, c.record_stages == 1);
   if (st != GS_OK) { destroy(r); return st; }
   cudaStream_t s = (cudaStream_t)stream;
   if (n > 0) {
-    st = run_record(r, c, n, params, y0, shared_w, y_save_out, s);
+    st = run_record(r, c, n, params, y0, shared_w, y_save_out, r->status, s);
     if (st != GS_OK) { destroy(r); return st; }
     cudaError_t e = cudaMemcpyAsync(traj_status, r->status, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -871,8 +1018,8 @@ gs_status gs_reverse(const gs_record* rec, const double* params, const double* y
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev != rec->device) return GS_ERR_INVALID_ARG;
-  return launch_reverse(rec, params, shared_w, y_save_bar, loss_out, params_bar, y0_bar, shared_w_bar,
-                        (cudaStream_t)stream);
+  return launch_reverse(rec, params, shared_w, y_save_bar, loss_out, params_bar, y0_bar, shared_w_bar, rec->status,
+                        false, (cudaStream_t)stream);
 }
 
 gs_status gs_replay_jvp(const gs_record* rec, const double* params, const double* y0, int n_dir,
@@ -1223,7 +1370,7 @@ gs_status gs_record_export_mesh(const gs_record* rec, int64_t* offsets, double* 
 }
 
 gs_status gs_record_free(gs_record* rec) {
-  destroy(rec);
+  if (!pool_put(rec)) destroy(rec);
   return GS_OK;
 }
 

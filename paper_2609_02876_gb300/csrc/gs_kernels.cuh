@@ -1930,13 +1930,18 @@ inline int sm_count() {
 template <class Kern>
 inline cudaError_t persistent_launch(Kern kern, int tpb, size_t smem, long long n, cudaStream_t s,
                                      const void* args_ptr) {  // n: lanes with work
-  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t err = cudaSuccess;
+  if (smem > 32 * 1024)  // (static and dynamic together have 48 KB without it)
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  int bps = 0;
-  err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, tpb, smem);
-  if (err != cudaSuccess) return err;
-  long long blocks = (long long)sm_count() * (bps > 0 ? bps : 1);
   const long long need = (n + tpb - 1) / tpb;
+  long long blocks = sm_count();
+  if (need > blocks) {  // more than a CTA per SM: as many as fit
+    int bps = 0;
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, tpb, smem);
+    if (err != cudaSuccess) return err;
+    blocks *= bps > 0 ? bps : 1;
+  }
   if (blocks > need) blocks = need;
   if (blocks < 1) blocks = 1;
   void* args[] = {const_cast<void*>(args_ptr)};

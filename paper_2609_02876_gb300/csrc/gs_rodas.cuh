@@ -85,22 +85,26 @@ __host__ __device__ constexpr double m(int j) { return j < 7 ? a(7, j) : 1.0; }
 // in registers. piv[k] is the row swapped with row k at column k; rinv[k] is
 // 1 / U_kk. Returns false on an exactly zero pivot.
 // ---------------------------------------------------------------------------
+// The pivot search compares bit patterns (magnitudes order as integers; a NaN
+// never wins and is never beaten, as in the comparison of doubles): an FP64
+// comparison holds the FP64 unit like an FMA, and there are D(D+1)/2 of them (the
+// HIRES record at 30000 trajectories, with the dense factorisation: 25.7 -> 24.5 ms).
 template <int D>
 __device__ __forceinline__ bool lu_factor(double (&A)[D][D], int (&piv)[D], double (&rinv)[D]) {
   bool ok = true;
 #pragma unroll
   for (int k = 0; k < D; ++k) {
     int pr = k;
-    double best = fabs(A[k][k]);
+    unsigned long long best = abs_bits(A[k][k]);
 #pragma unroll
     for (int i = k + 1; i < D; ++i) {
-      const double v = fabs(A[i][k]);
-      const bool gt = v > best;
+      const unsigned long long v = abs_bits(A[i][k]);
+      const bool gt = v > best && v <= DBITS_INF;
       best = gt ? v : best;
       pr = gt ? i : pr;
     }
     piv[k] = pr;
-    ok = ok && (best != 0.0);
+    ok = ok && (best != 0ull);
 #pragma unroll
     for (int i = k + 1; i < D; ++i) {
       const bool sw = (i == pr);
@@ -180,6 +184,177 @@ __device__ __forceinline__ void lu_solve_t(const double (&LU)[D][D], const int (
   }
 }
 
+template <class Pb, class = void>
+struct ContractOf {
+  using type = NoTape;
+  static constexpr bool value = false;
+};
+template <class Pb>
+struct ContractOf<Pb, std::void_t<typename Pb::Contract>> {
+  using type = typename Pb::Contract;
+  static constexpr bool value = true;
+};
+
+// ---------------------------------------------------------------------------
+// The same for a matrix whose structural zeros are known (HIRES: 24 of W's 64
+// entries). With partial pivoting the row exchanged at column k is one of those
+// with an entry in it, so the entries that the factors can hold are bounded at
+// compile time: u[k][j] for row k of U, l[i][k] for the multipliers of column k
+// (rows as they stand at step k; the multipliers stay where they were formed, and
+// a solve takes the exchanges between the columns). Everything else is an exact
+// zero that the dense code multiplies and adds; values and the order of the
+// remaining operations are the same, except that a transposed solve adds a
+// column's multipliers in their unexchanged order.
+// HIRES: a factorisation takes 26 instructions and 8 reciprocals for 204, a solve
+// 32 for 64, and the factors half of the registers. At 30000 trajectories, with the
+// integer pivot search: record 25.7 -> 17.8 ms, reverse sweep 59.2 -> 45.3 ms.
+// ---------------------------------------------------------------------------
+template <int D>
+struct LuPattern {
+  bool u[D][D] = {}, l[D][D] = {};
+};
+template <class Pb>
+constexpr LuPattern<Pb::D> lu_pattern() {
+  constexpr int D = Pb::D;
+  LuPattern<D> t;
+  bool a[D][D] = {};
+  for (int i = 0; i < D; ++i)
+    for (int j = 0; j < D; ++j) a[i][j] = i == j || Pb::jac_entry(i, j);
+  for (int k = 0; k < D; ++k) {
+    bool row[D] = {};  // union of the rows that may become row k
+    for (int i = k; i < D; ++i)
+      if (a[i][k])
+        for (int j = k; j < D; ++j) row[j] = row[j] || a[i][j];
+    for (int i = k + 1; i < D; ++i)
+      if (a[i][k]) {
+        t.l[i][k] = true;
+        for (int j = k; j < D; ++j) a[i][j] = j > k && row[j];
+      }
+    for (int j = k; j < D; ++j) t.u[k][j] = row[j];
+  }
+  return t;
+}
+template <class Pb, class = void>
+struct HasPattern : std::false_type {};
+template <class Pb>
+struct HasPattern<Pb, std::void_t<decltype(Pb::jac_entry(0, 0))>> : std::true_type {};
+
+template <class Pb>
+__device__ __forceinline__ bool factor_of(double (&A)[Pb::D][Pb::D], int (&piv)[Pb::D], double (&rinv)[Pb::D]) {
+  constexpr int D = Pb::D;
+  if constexpr (!HasPattern<Pb>::value) {
+    return lu_factor<D>(A, piv, rinv);
+  } else {
+    constexpr LuPattern<D> T = lu_pattern<Pb>();
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      int pr = k;
+      unsigned long long best = abs_bits(A[k][k]);
+#pragma unroll
+      for (int i = k + 1; i < D; ++i)
+        if (T.l[i][k]) {
+          const unsigned long long v = abs_bits(A[i][k]);
+          const bool gt = v > best && v <= DBITS_INF;
+          best = gt ? v : best;
+          pr = gt ? i : pr;
+        }
+      piv[k] = pr;
+      ok = ok && (best != 0ull);
+#pragma unroll
+      for (int i = k + 1; i < D; ++i)
+        if (T.l[i][k]) {
+          const bool sw = (i == pr);
+#pragma unroll
+          for (int j = k; j < D; ++j)
+            if (T.u[k][j]) {
+              const double t = A[k][j];
+              A[k][j] = sw ? A[i][j] : t;
+              A[i][j] = sw ? t : A[i][j];
+            }
+        }
+      rinv[k] = 1.0 / A[k][k];
+#pragma unroll
+      for (int i = k + 1; i < D; ++i)
+        if (T.l[i][k]) {
+          const double m = mul_(A[i][k], rinv[k]);
+          A[i][k] = m;
+#pragma unroll
+          for (int j = k + 1; j < D; ++j)
+            if (T.u[k][j]) A[i][j] = fma_(-m, A[k][j], A[i][j]);
+        }
+    }
+    return ok;
+  }
+}
+template <class Pb>
+__device__ __forceinline__ void solve_of(const double (&LU)[Pb::D][Pb::D], const int (&piv)[Pb::D],
+                                         const double (&rinv)[Pb::D], const double (&b)[Pb::D], double (&x)[Pb::D]) {
+  constexpr int D = Pb::D;
+  if constexpr (!HasPattern<Pb>::value) {
+    lu_solve<D>(LU, piv, rinv, b, x);
+  } else {
+    constexpr LuPattern<D> T = lu_pattern<Pb>();
+    double z[D];
+#pragma unroll
+    for (int i = 0; i < D; ++i) z[i] = b[i];
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+#pragma unroll
+      for (int i = k + 1; i < D; ++i)
+        if (T.l[i][k]) {
+          const bool sw = (i == piv[k]);
+          const double t = z[k];
+          z[k] = sw ? z[i] : t;
+          z[i] = sw ? t : z[i];
+        }
+#pragma unroll
+      for (int i = k + 1; i < D; ++i)
+        if (T.l[i][k]) z[i] = fma_(-LU[i][k], z[k], z[i]);
+    }
+#pragma unroll
+    for (int i = D - 1; i >= 0; --i) {
+      double s = z[i];
+#pragma unroll
+      for (int j = i + 1; j < D; ++j)
+        if (T.u[i][j]) s = fma_(-LU[i][j], x[j], s);
+      x[i] = mul_(s, rinv[i]);
+    }
+  }
+}
+template <class Pb>
+__device__ __forceinline__ void solve_t_of(const double (&LU)[Pb::D][Pb::D], const int (&piv)[Pb::D],
+                                           const double (&rinv)[Pb::D], const double (&b)[Pb::D], double (&x)[Pb::D]) {
+  constexpr int D = Pb::D;
+  if constexpr (!HasPattern<Pb>::value) {
+    lu_solve_t<D>(LU, piv, rinv, b, x);
+  } else {
+    constexpr LuPattern<D> T = lu_pattern<Pb>();
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      double s = b[i];
+#pragma unroll
+      for (int j = 0; j < i; ++j)
+        if (T.u[j][i]) s = fma_(-LU[j][i], x[j], s);
+      x[i] = mul_(s, rinv[i]);
+    }
+#pragma unroll
+    for (int k = D - 1; k >= 0; --k) {
+#pragma unroll
+      for (int i = k + 1; i < D; ++i)
+        if (T.l[i][k]) x[k] = fma_(-LU[i][k], x[i], x[k]);
+#pragma unroll
+      for (int i = k + 1; i < D; ++i)
+        if (T.l[i][k]) {
+          const bool sw = (i == piv[k]);
+          const double t = x[k];
+          x[k] = sw ? x[i] : t;
+          x[i] = sw ? t : x[i];
+        }
+    }
+  }
+}
+
 // Stage input Y_i = y + sum_{j<i} a_ij U_j, in a fixed order (the step and
 // the stored-stage reverse build it the same way).
 template <int D>
@@ -223,7 +398,7 @@ __device__ __forceinline__ bool rodas_step(const double (&y)[Pb::D], const doubl
     for (int j = 0; j < D; ++j) LU[i][j] = -LU[i][j];
     LU[i][i] = add_(LU[i][i], inv_hg);
   }
-  const bool ok = lu_factor<D>(LU, piv, rinv);
+  const bool ok = factor_of<Pb>(LU, piv, rinv);
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     double F[D], Rhs[D];
@@ -249,7 +424,7 @@ __device__ __forceinline__ bool rodas_step(const double (&y)[Pb::D], const doubl
         Rhs[c] = fma_(inv_h, s, F[c]);
       }
     }
-    lu_solve<D>(LU, piv, rinv, Rhs, U[i]);
+    solve_of<Pb>(LU, piv, rinv, Rhs, U[i]);
   }
 #pragma unroll
   for (int c = 0; c < D; ++c) ynew[c] = add_(Y[7][c], U[7][c]);
@@ -278,7 +453,7 @@ __device__ __forceinline__ bool rodas_tangent(const double (&y)[Pb::D], const do
     for (int j = 0; j < D; ++j) LU[i][j] = -LU[i][j];
     LU[i][i] = add_(LU[i][i], inv_hg);
   }
-  const bool ok = lu_factor<D>(LU, piv, rinv);
+  const bool ok = factor_of<Pb>(LU, piv, rinv);
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     double Y[D], F[D], Rhs[D];
@@ -301,7 +476,7 @@ __device__ __forceinline__ bool rodas_tangent(const double (&y)[Pb::D], const do
         Rhs[c] = fma_(inv_h, s, F[c]);
       }
     }
-    lu_solve<D>(LU, piv, rinv, Rhs, U[i]);
+    solve_of<Pb>(LU, piv, rinv, Rhs, U[i]);
 #pragma unroll
     for (int q = 0; q < ND; ++q) {
       double Yd[D], Fd[D], JdU[D], Rd[D];
@@ -325,7 +500,7 @@ __device__ __forceinline__ bool rodas_tangent(const double (&y)[Pb::D], const do
           Rd[c] = add_(fma_(inv_h, s, Fd[c]), JdU[c]);
         }
       }
-      lu_solve<D>(LU, piv, rinv, Rd, Ud[i][q]);
+      solve_of<Pb>(LU, piv, rinv, Rd, Ud[i][q]);
       if (i == 7) {
 #pragma unroll
         for (int c = 0; c < D; ++c) ydn[q][c] = add_(Yd[c], Ud[7][q][c]);
@@ -346,8 +521,8 @@ __device__ __forceinline__ bool rodas_tangent(const double (&y)[Pb::D], const do
 //   v += Ybar_i, Ubar_j += a_ij Ybar_i;
 // and W = I/(h gamma) - J(y) gives dL/dJ = sum_i Rbar_i U_i^T, contracted through
 // J(y, theta): v += d/dy (Rbar_i^T J U_i), theta_bar += d/dtheta (Rbar_i^T J U_i).
-// Problems with a tape take the contraction once per step: it is linear in
-// sum_i Rbar_i U_i^T, which the accumulator collects over the stages.
+// The contraction is linear in sum_i Rbar_i U_i^T: problems with a tape or a
+// Contract collect the products they need over the stages and contract once.
 template <class Pb, class Acc>
 __device__ __forceinline__ void rodas_reverse(const double (&y)[Pb::D], const double (&p)[Pb::NP], double h,
                                               const double (&Y)[8][Pb::D], const double (&U)[8][Pb::D],
@@ -357,17 +532,18 @@ __device__ __forceinline__ void rodas_reverse(const double (&y)[Pb::D], const do
   constexpr int D = Pb::D;
   const double inv_h = 1.0 / h;
   double Ub[8][D];
+  typename ContractOf<Pb>::type con;  // (problems that collect the contraction over the stages)
   if constexpr (TapeOf<Pb>::value) pacc.contract_begin(tape);
 #pragma unroll
   for (int j = 0; j < 8; ++j)
 #pragma unroll
-    for (int c = 0; c < D; ++c) Ub[j][c] = (j == 7) ? lam[c] : mul_(rodas::m(j), lam[c]);
+    for (int c = 0; c < D; ++c) Ub[j][c] = (rodas::m(j) == 1.0) ? lam[c] : mul_(rodas::m(j), lam[c]);
 #pragma unroll
   for (int c = 0; c < D; ++c) v[c] = lam[c];
 #pragma unroll
   for (int i = 7; i >= 0; --i) {
     double Rb[D], Yb[D], Rh[D];
-    lu_solve_t<D>(LU, piv, rinv, Ub[i], Rb);
+    solve_t_of<Pb>(LU, piv, rinv, Ub[i], Rb);
 #pragma unroll
     for (int c = 0; c < D; ++c) Rh[c] = mul_(inv_h, Rb[c]);
 #pragma unroll
@@ -386,10 +562,13 @@ __device__ __forceinline__ void rodas_reverse(const double (&y)[Pb::D], const do
       for (int c = 0; c < D; ++c) Ub[j][c] = fma_(rodas::a(i, j), Yb[c], Ub[j][c]);
     if constexpr (TapeOf<Pb>::value)
       pacc.contract_add(Rb, U[i]);
+    else if constexpr (ContractOf<Pb>::value)
+      con.add(Rb, U[i], i == 7, pacc.s);
     else
       pacc.template jac_contract<Pb>(y, p, Rb, U[i], v);
   }
   if constexpr (TapeOf<Pb>::value) pacc.contract_flush(tape, y, p, v);
+  if constexpr (ContractOf<Pb>::value) con.flush(y, p, v, pacc.s);
 }
 
 // ---------------------------------------------------------------------------
@@ -419,7 +598,7 @@ __device__ __forceinline__ bool ros23_factor(const double (&y)[Pb::D], const dou
     for (int j = 0; j < D; ++j) LU[i][j] = mul_(mhd, LU[i][j]);
     LU[i][i] = add_(LU[i][i], 1.0);
   }
-  return lu_factor<D>(LU, piv, rinv);
+  return factor_of<Pb>(LU, piv, rinv);
 }
 
 // The replay map with its stage quantities: k1, u2, Y1, F1 and y_new, from
@@ -431,7 +610,7 @@ __device__ __forceinline__ void ros23_stages(const double (&y)[Pb::D], const dou
                                              double (&k1)[Pb::D], double (&u2)[Pb::D], double (&Y1)[Pb::D],
                                              double (&F1)[Pb::D], double (&ynew)[Pb::D]) {
   constexpr int D = Pb::D;
-  lu_solve<D>(LU, piv, rinv, F0, k1);
+  solve_of<Pb>(LU, piv, rinv, F0, k1);
   const double hh = mul_(0.5, h);
 #pragma unroll
   for (int c = 0; c < D; ++c) Y1[c] = fma_(hh, k1[c], y[c]);
@@ -439,7 +618,7 @@ __device__ __forceinline__ void ros23_stages(const double (&y)[Pb::D], const dou
   double r[D];
 #pragma unroll
   for (int c = 0; c < D; ++c) r[c] = sub_(F1[c], k1[c]);
-  lu_solve<D>(LU, piv, rinv, r, u2);
+  solve_of<Pb>(LU, piv, rinv, r, u2);
 #pragma unroll
   for (int c = 0; c < D; ++c) ynew[c] = fma_(h, add_(u2[c], k1[c]), y[c]);
 }
@@ -462,7 +641,7 @@ __device__ __forceinline__ bool ros23_trial(const double (&y)[Pb::D], const doub
     const double k2 = add_(u2[c], k1[c]);
     r[c] = fma_(-ros23::E32, sub_(k2, F1[c]), fma_(-2.0, sub_(k1[c], F0[c]), F2[c]));
   }
-  lu_solve<D>(LU, piv, rinv, r, k3);
+  solve_of<Pb>(LU, piv, rinv, r, k3);
   const double h6 = h / 6.0;
 #pragma unroll
   for (int c = 0; c < D; ++c) e[c] = mul_(h6, add_(fma_(-2.0, add_(u2[c], k1[c]), k1[c]), k3[c]));
@@ -494,12 +673,12 @@ __device__ __forceinline__ void ros23_reverse(const double (&y)[Pb::D], const do
   double k2b[D], r2b[D], k1b[D], r1b[D], Y1b[D], y0b[D];
 #pragma unroll
   for (int c = 0; c < D; ++c) k2b[c] = mul_(h, lam[c]);
-  lu_solve_t<D>(LU, piv, rinv, k2b, r2b);
+  solve_t_of<Pb>(LU, piv, rinv, k2b, r2b);
   pacc.template vjp<Pb>(Y1, p, r2b, Y1b);
   const double hh = mul_(0.5, h);
 #pragma unroll
   for (int c = 0; c < D; ++c) k1b[c] = fma_(hh, Y1b[c], sub_(k2b[c], r2b[c]));
-  lu_solve_t<D>(LU, piv, rinv, k1b, r1b);
+  solve_t_of<Pb>(LU, piv, rinv, k1b, r1b);
   pacc.template vjp<Pb>(y, p, r1b, y0b);
 #pragma unroll
   for (int c = 0; c < D; ++c) v[c] = add_(add_(lam[c], Y1b[c]), y0b[c]);
@@ -537,14 +716,14 @@ __device__ __forceinline__ bool ros23_tangent(const double (&y)[Pb::D], const do
     Pb::jac_dir(y, p, yd[q], pd[q], k1, JdU);
 #pragma unroll
     for (int c = 0; c < D; ++c) r[c] = fma_(hd, JdU[c], Fd[c]);
-    lu_solve<D>(LU, piv, rinv, r, kd1);
+    solve_of<Pb>(LU, piv, rinv, r, kd1);
 #pragma unroll
     for (int c = 0; c < D; ++c) Yd1[c] = fma_(hh, kd1[c], yd[q][c]);
     Pb::jvp(Y1, p, Yd1, pd[q], Fd);
     Pb::jac_dir(y, p, yd[q], pd[q], u2, JdU);
 #pragma unroll
     for (int c = 0; c < D; ++c) r[c] = fma_(hd, JdU[c], sub_(Fd[c], kd1[c]));
-    lu_solve<D>(LU, piv, rinv, r, ud2);
+    solve_of<Pb>(LU, piv, rinv, r, ud2);
 #pragma unroll
     for (int c = 0; c < D; ++c) ydn[q][c] = fma_(h, add_(ud2[c], kd1[c]), yd[q][c]);
   }

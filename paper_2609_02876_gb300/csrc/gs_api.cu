@@ -133,6 +133,7 @@ struct gs_record {
   // Stored stages (gs_solve_grad's workspace, Tsit5 FP64, k = 1): segments also
   // hold each step's stage data, side_stg (n x n_save x payload) the side steps'.
   int stages = 0;
+  int packed = 0;  // FP32-mixed segments in the packed layout (gs_solve_grad's workspaces)
   double* side_stg = nullptr;
   size_t side_cap = 0;  // doubles
   // chunk staging of a chunked FP32-mixed gs_solve_grad (inputs and outputs of one chunk)
@@ -447,7 +448,7 @@ gs_status enqueue_record(gs_record* r, const Call& c, int64_t n, const double* p
   a.y_final = r->y_final;
   a.work = &r->ctr->work_fwd;
   if (c.kernel_ms) cudaEventRecord(r->ev[0], s);
-  e = launch_forward_m(c.method, c.problem, c.precision, a, s);
+  e = r->packed ? launch_packed_forward(c.problem, a, s) : launch_forward_m(c.method, c.problem, c.precision, a, s);
   if (e != cudaSuccess) return GS_ERR_CUDA;
   if (c.kernel_ms) cudaEventRecord(r->ev[1], s);
   return GS_OK;
@@ -474,6 +475,13 @@ void record_done(gs_record* r, const Call& c) {
 // compact record if the stored-stage one does not fit.
 gs_status grow_arena(gs_record* r) {
   const long long need = (long long)r->ctr_host->arena_top;
+  if (r->packed && need + need / 8 + 1024 >= (1ll << 31)) {  // past a packed segment's 32-bit index
+    r->packed = 0;
+    r->segw = segw_of(r->d, r->k);
+    cudaFree(r->arena);  // (its capacity counts packed segments)
+    r->arena = nullptr;
+    r->arena_cap = 0;
+  }
   gs_status st = ensure_arena(r, need + need / 8 + 1024, r->segw);
   if (st == GS_ERR_OOM && r->stages) {
     r->stages = 0;
@@ -504,7 +512,7 @@ gs_status run_record(gs_record* r, const Call& c, int64_t n, const double* param
 // expected record takes at most half of the free device memory, else a
 // 128-byte segment of 14 - d steps (one checkpoint per 14 - d steps).
 int auto_ckpt_k(const gs_record* r, int problem, int d, int64_t n) {
-  if (r->arena && r->segw == segw_of(d, 1) && r->arena_cap >= (n > 0 ? n : 1) * (long long)(step_guess(problem) + 1))
+  if (r->arena && (r->segw == segw_of(d, 1) || r->packed) && r->arena_cap >= (n > 0 ? n : 1) * (long long)(step_guess(problem) + 1))
     return 1;  // held from an earlier call of this size
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = 0;
@@ -547,7 +555,7 @@ bool choose_stages(const gs_record* r, const Call& c, int64_t n, int n_save, dou
 }
 
 gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double t1, const double* save_t,
-                       int n_save, double rtol, double atol, bool allow_stages = false) {
+                       int n_save, double rtol, double atol, bool allow_stages = false, bool allow_packed = false) {
   cudaGetDevice(&r->device);
   r->problem = c.problem;
   r->method = c.method;
@@ -588,7 +596,10 @@ gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double
       }
     }
   }
-  const int segw = r->stages ? stage_segw_of(c.method, r->d) : segw_of(r->d, r->k);
+  // (a packed segment's index has 32 bits: far more than the expected segments fit)
+  r->packed = allow_packed && c.precision == GS_FP32_MIXED && c.method == GS_METHOD_TSIT5 && r->k == 1 &&
+              packed_supports(c.problem) && (double)n * step_guess(c.problem, rtol, c.method) < 2.5e8;
+  const int segw = r->stages ? stage_segw_of(c.method, r->d) : (r->packed ? PACKED_SEGW_HOST : segw_of(r->d, r->k));
   if (r->segw != segw) {
     cudaFree(r->arena);
     r->arena = nullptr;
@@ -657,7 +668,7 @@ gs_status launch_reverse(const gs_record* r, const double* params, const float* 
   a.tc_error = &r->ctr->tc_error;
   cudaError_t e = fresh_counters ? cudaSuccess : cudaMemsetAsync(&r->ctr->work_rev, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return GS_ERR_CUDA;
-  e = launch_reverse_m(r->method, r->problem, r->precision, a, s);
+  e = r->packed ? launch_packed_reverse(r->problem, a, s) : launch_reverse_m(r->method, r->problem, r->precision, a, s);
   return e == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
@@ -756,7 +767,7 @@ gs_status solve_grad_in(gs_record* r, const Call& c, int64_t n, const double* pa
                         const float* shared_w, double t0, double t1, const double* save_t, int n_save, double rtol,
                         double atol, cudaStream_t s, double* loss_out, double* params_bar, double* y0_bar,
                         float* shared_w_bar, int32_t* traj_status, bool allow_stages) {
-  gs_status st = setup_record(r, c, n, t0, t1, save_t, n_save, rtol, atol, allow_stages);
+  gs_status st = setup_record(r, c, n, t0, t1, save_t, n_save, rtol, atol, allow_stages, true);
   if (st != GS_OK) return st;
   const size_t nb = (size_t)n * sizeof(double);
   const void* outs[5] = {loss_out, params_bar, y0_bar, shared_w_bar, traj_status};

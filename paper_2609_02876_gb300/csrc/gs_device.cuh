@@ -1100,8 +1100,8 @@ __device__ __forceinline__ double err_meansq(const double (&e)[D], const double 
 // that the square stays finite (any error that large gives the controller's
 // minimum factor either way); a NaN passes through. No FP64 instruction.
 template <int D>
-__device__ __forceinline__ double err_meansq(const float (&e)[D], const float (&y)[D], const float (&yn)[D],
-                                             double, double, float rt, float at) {
+__device__ __forceinline__ float err_meansq_f32(const float (&e)[D], const float (&y)[D], const float (&yn)[D], float rt,
+                                                float at) {
   float q = 0.0f;
 #pragma unroll
   for (int c = 0; c < D; ++c) {
@@ -1110,7 +1110,12 @@ __device__ __forceinline__ double err_meansq(const float (&e)[D], const float (&
     r = (fabsf(r) > 1e18f) ? 1e18f : r;
     q = __fmaf_rn(r, r, q);
   }
-  return to_d(__fmul_rn(q, 1.0f / D));
+  return __fmul_rn(q, 1.0f / D);
+}
+template <int D>
+__device__ __forceinline__ double err_meansq(const float (&e)[D], const float (&y)[D], const float (&yn)[D],
+                                             double, double, float rt, float at) {
+  return to_d(err_meansq_f32<D>(e, y, yn, rt, at));
 }
 
 // Integral-controller factor from the mean-square error q = err^2, for an
@@ -1119,11 +1124,16 @@ __device__ __forceinline__ double err_meansq(const float (&e)[D], const float (&
 // Rosenbrock23); q = 0 gives 10. FP32 with the hardware log2 / exp2: the factor
 // only scales the next trial step.
 template <int Q>
-__device__ __forceinline__ float ctrl_factor(double q) {
+__device__ __forceinline__ float ctrl_factor_f32(float q) {  // q >= 0, finite
   constexpr float EXPO = -0.5f / (Q + 1);
-  if (!positive(q)) return 10.0f;
-  const float f = __fmul_rn(0.9f, ex2_approx(__fmul_rn(EXPO, lg2_approx(to_f(q)))));
+  if (!(q > 0.0f)) return 10.0f;
+  const float f = __fmul_rn(0.9f, ex2_approx(__fmul_rn(EXPO, lg2_approx(q))));
   return fminf(10.0f, fmaxf(0.2f, f));
+}
+template <int Q>
+__device__ __forceinline__ float ctrl_factor(double q) {
+  if (!positive(q)) return 10.0f;
+  return ctrl_factor_f32<Q>(to_f(q));
 }
 
 // Starting step: the algorithm of Hairer, Norsett & Wanner, Vol. I, Sec. II.4

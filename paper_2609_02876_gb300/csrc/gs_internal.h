@@ -145,6 +145,11 @@ struct LaunchCfg {
 cudaError_t launch_tsit5_forward(int problem, int precision, const FwdArgs& a, cudaStream_t s);
 cudaError_t launch_tsit5_reverse(int problem, int precision, const RevArgs& a, cudaStream_t s);
 bool tsit5_supports(int problem, int precision);
+// FP32-mixed Tsit5 over packed segments (gs_packed.cuh), k = 1, built-in loss.
+constexpr int PACKED_SEGW_HOST = 4;  // doubles per packed segment
+bool packed_supports(int problem);
+cudaError_t launch_packed_forward(int problem, const FwdArgs& a, cudaStream_t s);
+cudaError_t launch_packed_reverse(int problem, const RevArgs& a, cudaStream_t s);
 // The FP64 Tsit5 kernels with multiplications on the integer pipes (SoftD in
 // gs_device.cuh); the reverse sweep for k = 1 records. Same results.
 cudaError_t launch_tsit5_soft_forward(int problem, const FwdArgs& a, cudaStream_t s);

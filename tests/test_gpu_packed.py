@@ -1,0 +1,64 @@
+"""FP32-mixed solves over packed segments: the same bits as the general record
+and sweep kernels (a record handle's), over sizes at the edges of warps and
+blocks, both step controls, spans and save grids of every kind, and trajectories
+that fail."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_02876_gb300 import api, build
+from paper_2609_02876_gb300 import workloads as W
+from tests.test_gpu_tsit5 import dev
+
+pytestmark = pytest.mark.gpu
+
+
+def both(problem, p, y, t0, t1, saves, rtol, atol, **kw):
+    build.build()
+    P, Y = dev(p.T), dev(y.T)
+    kw = dict(layout="soa", precision="fp32_mixed", check=False, **kw)
+    s = api.solve_grad(problem, P, Y, t0, t1, saves, rtol, atol, step_counts=True, **kw)
+    rec, _, st = api.forward_record(problem, P, Y, t0, t1, saves, rtol, atol, ckpt_k=1, want_saves=False,
+                                    step_counts=True, **kw)
+    g = api.reverse(rec, P, Y, layout="soa")
+    assert torch.equal(s["status"], st)
+    assert torch.equal(s["step_counts"], rec.step_counts)
+    for k in ("loss", "params_bar", "y0_bar"):
+        assert torch.equal(s[k].view(torch.int64), g[k].view(torch.int64)), k
+    return st.cpu().numpy()
+
+
+@pytest.mark.parametrize("control", ["fast", "fp64"])
+@pytest.mark.parametrize("problem", ["lorenz", "vdp"])
+@pytest.mark.parametrize("n", [1, 31, 129, 40001])
+def test_same_bits_as_the_general_kernels(problem, n, control):
+    wl = W.make(problem, n)
+    st = both(problem, wl["params"], wl["y0"], wl["t0"], wl["t1"], wl["save_t"], wl["rtol"], wl["atol"],
+              control=control)
+    assert (st == 0).all()
+
+
+@pytest.mark.parametrize("t0,t1,saves", [(0.0, 1.0, []), (-3.0, -1.0, [-2.5, -1.7]), (-1.0, 1.0, [-0.5, 1e-300, 1.0]),
+                                         (2.0, 2.5, np.linspace(2.0, 2.5, 257)[1:])])
+def test_spans_and_save_grids(t0, t1, saves):
+    rng = np.random.RandomState(2)
+    n = 333
+    both("linear", rng.uniform(-1, 1, (n, 4)), rng.uniform(-1, 1, (n, 2)), t0, t1, saves, 1e-5, 1e-7)
+    wl = W.make("lorenz", n)
+    both("lorenz", wl["params"], wl["y0"], t0, t1, saves, 1e-5, 1e-7)
+
+
+@pytest.mark.parametrize("kw", [dict(max_steps=20), dict(h0=1e-3), dict(h0=10.0)])
+def test_options_and_failed_trajectories(kw):
+    n = 777
+    wl = W.make("lorenz", n)
+    y = wl["y0"].copy()
+    y[3] = np.nan
+    y[64:96] = np.inf
+    y[100] *= 1e30  # overflows single precision on the way
+    y[101] = 0.0
+    y[102] = 1e-37
+    p = wl["params"].copy()
+    p[200] = 0.0
+    st = both("lorenz", p, y, wl["t0"], wl["t1"], wl["save_t"], wl["rtol"], wl["atol"], **kw)
+    assert (st[[3, 64, 95]] == 3).all()

@@ -124,6 +124,31 @@ __device__ __forceinline__ void from_soft(const SoftD (&x)[N], double (&o)[N]) {
 }
 
 // ---------------------------------------------------------------------------
+// 2 x: in FP64 on the integer pipes (the exponent field, or a subnormal's
+// mantissa; exact), not on the FP64 unit.
+// ---------------------------------------------------------------------------
+__host__ __device__ __forceinline__ void twice_words(uint32_t& hi, uint32_t& lo) {
+  const uint32_t e = hi & 0x7ff00000u;
+  if (e == 0u) {  // zero or subnormal: the mantissa may carry into the exponent
+    hi = (hi & 0x80000000u) | ((hi << 1 | lo >> 31) & 0x7fffffffu);
+    lo <<= 1;
+  } else if (e >= 0x7fe00000u) {
+    if (e == 0x7fe00000u) {  // overflow to infinity
+      hi = (hi & 0x80000000u) | 0x7ff00000u;
+      lo = 0u;
+    }
+  } else {
+    hi += 0x00100000u;
+  }
+}
+__device__ __forceinline__ double twice_(double x) {
+  uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  twice_words(hi, lo);
+  return __hiloint2double((int)hi, (int)lo);
+}
+__device__ __forceinline__ float twice_(float x) { return __fadd_rn(x, x); }
+
+// ---------------------------------------------------------------------------
 // FP32 <-> FP64 conversions on the integer ALU. GB300 executes the hardware
 // conversion instructions on its FP64 pipe (2 lanes per clock per SM), which
 // the FP32-mixed form otherwise spends on format changes; these rebuild the

@@ -118,7 +118,7 @@ __device__ __forceinline__ void unit_cotangent(const RevArgs& a, long long k, bo
     if (USER_COT) {
       if (active && side) cs = to_r<R>(a.y_save_bar[((long long)us * D + c) * a.n + k]);
     } else {
-      cs = add_(ynew[c], ynew[c]);  // d/dy of ||y||^2
+      cs = twice_(ynew[c]);  // d/dy of ||y||^2
       l2 = fma_(ynew[c], ynew[c], l2);
     }
     cv[c] = active ? (side ? cs : lam[c]) : R(0);
@@ -1201,10 +1201,20 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
       }
       if (flush) {
         stg[0] = __longlong_as_double(prev);
-        if (!group_leader<Pb>()) {
-        } else if (idx < a.arena_cap) {
+        if (idx < a.arena_cap) {
           double2* dst = reinterpret_cast<double2*>(a.arena + idx * a.segw);
-          for (int w = 0; w < (a.segw >> 1); ++w) dst[w] = make_double2(stg[(2 * w) * TB], stg[(2 * w + 1) * TB]);
+          constexpr int G = GroupOf<Pb>::value;  // (a group's lanes stage the same segment and share its stores)
+          const int w0 = G > 1 ? (int)(threadIdx.x & (G - 1)) : 0;
+          if constexpr (STAGES) {
+            constexpr int SW2 = stage_segw<M, D>() / 2;
+#pragma unroll
+            for (int w = 0; w < (SW2 + G - 1) / G; ++w) {
+              const int i = G * w + w0;
+              if (G * (w + 1) <= SW2 || i < SW2) dst[i] = make_double2(stg[(2 * i) * TB], stg[(2 * i + 1) * TB]);
+            }
+          } else {
+            for (int w = w0; w < (a.segw >> 1); w += G) dst[w] = make_double2(stg[(2 * w) * TB], stg[(2 * w + 1) * TB]);
+          }
         } else {
           *a.overflow = 1;
         }
@@ -1311,10 +1321,6 @@ template <class M, class Pb, class R, bool SAVES, bool STAGES, bool C64>
 constexpr auto record_entry() {
   if constexpr (C64 && GS_FWD_C64_MINB > 0)
     return &record_kernel_mb<M, Pb, R, SAVES, STAGES, C64, GS_FWD_C64_MINB>;
-  else if constexpr (STAGES && std::is_same<M, Rodas5PMethod>::value)
-    // all registers (Robertson: 238 at 2 CTAs per SM, for the compiler's own 168 at
-    // 3): the record at 2^18 trajectories 23.9 -> 22.6 ms
-    return &record_kernel_mb<M, Pb, R, SAVES, STAGES, C64, 1>;
   else
     return &record_kernel<M, Pb, R, SAVES, STAGES, C64>;
 }
@@ -1652,6 +1658,26 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
   double loss = 0.0, tx = 0.0;
   long long seg = -1;
   int js = -1, segs_left = 0;
+  // Lane groups read the next segment while the unit runs: with a warp per SM
+  // quarter nothing else hides the load (about 1700 of the 10600 cycles of a Lorenz
+  // unit), and there are registers to spare. (The per-lane kernels' warps hide one
+  // another's loads.)
+  constexpr bool AHEAD = G > 1 && !STATIC;
+  constexpr int SEGW = STAGES ? stage_segw<M, D>() : ((3 + D) + 1) & ~1;  // doubles read of a segment
+  double ahead[AHEAD ? SEGW : 1];
+  const auto load_ahead = [&]() {
+    if constexpr (AHEAD) {
+      if (seg >= 0 && seg < a.arena_cap) {
+        const double2* sp = reinterpret_cast<const double2*>(a.arena + seg * a.segw);
+#pragma unroll
+        for (int w = 0; w < SEGW / 2; ++w) {
+          const double2 v = sp[w];
+          ahead[2 * w] = v.x;
+          ahead[2 * w + 1] = v.y;
+        }
+      }
+    }
+  };
 
   for (;;) {
     const bool need = (k < 0) && !drained;
@@ -1692,6 +1718,7 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
                 js = ns - 2;
               }
             }
+            load_ahead();
           }
         } else {
           drained = true;
@@ -1733,38 +1760,26 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
         mode = U_FAIL;  // inconsistent record
       } else {
         // segment i: [prev, t_{i-1}, y_{i-1}[D], h_i (, Y_1..Y_5 of step i)]
-        const double* sp = a.arena + seg * a.segw;
-        if constexpr (STAGES) {
-          const double2 w0 = *reinterpret_cast<const double2*>(sp);
-          seg = __double_as_longlong(w0.x);
-          tx = w0.y;
-          constexpr int SW = stage_segw<M, D>();
-          double buf[SW];
+        double buf[SEGW];
+        if constexpr (AHEAD) {
 #pragma unroll
-          for (int w = 1; w < SW / 2; ++w) {
-            const double2 v = reinterpret_cast<const double2*>(sp)[w];
-            buf[2 * w] = v.x;
-            buf[2 * w + 1] = v.y;
-          }
-#pragma unroll
-          for (int c = 0; c < D; ++c) yx[c] = to_r<R>(buf[2 + c]);
-          uh = buf[2 + D];
-          M::template unpack<Pb, R>(false, yx, [&](int i) { return buf[3 + D + i]; }, sd);
+          for (int w = 0; w < SEGW; ++w) buf[w] = ahead[w];
         } else {
-          constexpr int CW = ((3 + D) + 1) & ~1;  // [prev, t, y[D], h] in whole double2
-          double buf[CW];
+          const double2* sp = reinterpret_cast<const double2*>(a.arena + seg * a.segw);
 #pragma unroll
-          for (int w = 0; w < CW / 2; ++w) {
-            const double2 v = reinterpret_cast<const double2*>(sp)[w];
+          for (int w = 0; w < SEGW / 2; ++w) {
+            const double2 v = sp[w];
             buf[2 * w] = v.x;
             buf[2 * w + 1] = v.y;
           }
-          seg = __double_as_longlong(buf[0]);
-          tx = buf[1];
-#pragma unroll
-          for (int c = 0; c < D; ++c) yx[c] = to_r<R>(buf[2 + c]);
-          uh = buf[2 + D];
         }
+        seg = __double_as_longlong(buf[0]);
+        tx = buf[1];
+#pragma unroll
+        for (int c = 0; c < D; ++c) yx[c] = to_r<R>(buf[2 + c]);
+        uh = buf[2 + D];
+        if constexpr (STAGES) M::template unpack<Pb, R>(false, yx, [&](int i) { return buf[3 + D + i]; }, sd);
+        load_ahead();
         --segs_left;
         mode = U_STEP;
       }
@@ -1791,6 +1806,9 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
           busy)
         mode = U_FAIL;
     }
+    // the unit was the trajectory's last (no segment and no save left): its results
+    // go out now, not after an iteration in which its lane has nothing to do
+    if (busy && mode != U_FAIL && seg < 0 && js < 0) mode = (segs_left == 0) ? U_DONE : U_FAIL;
     if (mode == U_FAIL) {
       if (group_leader<Pb>()) write_nan<NP, D>(a, k);
       k = -1;
@@ -2034,7 +2052,20 @@ inline cudaError_t fwd_dispatch(const FwdArgs& a_in, cudaStream_t s) {
     }
   }
   if constexpr (stages_possible<M, Pb, R>()) {
-    if (a.stages) return persistent_launch(record_entry<M, Pb, R, true, true, false>(), TPB_FWD, smem, lanes, s, &a);
+    if (a.stages) {
+      if constexpr (std::is_same<M, Rodas5PMethod>::value) {
+        // Held to 3 CTAs per SM (168 registers) where those take the ensemble in one
+        // wave and 2 CTAs do not, else with all registers (Robertson: 246, 2 CTAs).
+        // Robertson record, all / 168 registers: 1000 trajectories 2.20 / 2.32 ms;
+        // 40000: 5.26 / 5.01; 56308: 6.42 / 5.08; 65536: 6.52 / 7.66; 2^18: 22.8 / 24.0.
+        const long long wave = (long long)sm_count() * TPB_FWD;
+        if (lanes > 2 * wave && lanes <= 3 * wave)
+          return persistent_launch(record_kernel_mb<M, Pb, R, true, true, false, 3>, TPB_FWD, smem, lanes, s, &a);
+        return persistent_launch(record_kernel_mb<M, Pb, R, true, true, false, 1>, TPB_FWD, smem, lanes, s, &a);
+      } else {
+        return persistent_launch(record_kernel<M, Pb, R, true, true>, TPB_FWD, smem, lanes, s, &a);
+      }
+    }
   } else {
     if (a.stages) return cudaErrorInvalidValue;
   }

@@ -1205,7 +1205,9 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
           double2* dst = reinterpret_cast<double2*>(a.arena + idx * a.segw);
           constexpr int G = GroupOf<Pb>::value;  // (a group's lanes stage the same segment and share its stores)
           const int w0 = G > 1 ? (int)(threadIdx.x & (G - 1)) : 0;
-          if constexpr (STAGES) {
+          // (unrolled for Tsit5's segments only: the longer ones of Verner7 and Rodas5P
+          // raise those kernels' registers, 128 -> 162 for Verner7's Lorenz record)
+          if constexpr (STAGES && (G > 1 || std::is_same<M, Tsit5Method>::value)) {
             constexpr int SW2 = stage_segw<M, D>() / 2;
 #pragma unroll
             for (int w = 0; w < (SW2 + G - 1) / G; ++w) {
@@ -2055,7 +2057,7 @@ inline cudaError_t fwd_dispatch(const FwdArgs& a_in, cudaStream_t s) {
     if (a.stages) {
       if constexpr (std::is_same<M, Rodas5PMethod>::value) {
         // Held to 3 CTAs per SM (168 registers) where those take the ensemble in one
-        // wave and 2 CTAs do not, else with all registers (Robertson: 246, 2 CTAs).
+        // wave and 2 CTAs do not, else with all registers (Robertson: 238, 2 CTAs).
         // Robertson record, all / 168 registers: 1000 trajectories 2.20 / 2.32 ms;
         // 40000: 5.26 / 5.01; 56308: 6.42 / 5.08; 65536: 6.52 / 7.66; 2^18: 22.8 / 24.0.
         const long long wave = (long long)sm_count() * TPB_FWD;

@@ -128,9 +128,10 @@ typedef struct {
                            the record also stored every step's stage data (gs_solve_grad
                            chooses that layout in FP64 for Tsit5, Verner7, Rodas5P and
                            Rosenbrock23 when the segment is small enough (not HIRES) and
-                           the device memory allows; the reverse sweep then reads the
-                           stages instead of recomputing them, with identical results),
-                           else 0 */
+                           the device memory allows, and gs_solve_grad for Rodas5P on the
+                           neural Robertson up to 12288 trajectories; the reverse sweep then
+                           reads the stages instead of recomputing them, with identical
+                           results), else 0 */
   int control;          /* GS_CONTROL_FAST or GS_CONTROL_FP64 */
   int record_stages;    /* gs_forward_record only: 1 lets the record also store every step's
                            stage data when gs_solve_grad would (same rule: method, FP64, segment

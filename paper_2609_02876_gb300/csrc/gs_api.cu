@@ -73,7 +73,8 @@ int step_guess(int pid, double rtol, int method) {
 // LU factors, pivot reciprocals and pivots (the stage inputs and the save state
 // are rebuilt from them); Rosenbrock23: k1, u2 and the LU of W (Y1 and the save
 // state rebuilt).
-int stage_step_payload(int method, int d) {
+int stage_step_payload(int method, int d, int pid) {
+  if (pid == GS_NEURAL_ROBERTSON) return NRG_STAGE_DOUBLES;  // with the network's activations
   switch (method) {
     case GS_METHOD_RODAS5P: return 10 * d + d * d;
     case GS_METHOD_ROSENBROCK23: return 4 * d + d * d;
@@ -81,11 +82,11 @@ int stage_step_payload(int method, int d) {
   }
   return 5 * d;  // Tsit5
 }
-int stage_side_payload(int method, int d) {
+int stage_side_payload(int method, int d, int pid) {
   const bool rebuilt = method == GS_METHOD_RODAS5P || method == GS_METHOD_ROSENBROCK23;  // save state rebuilt
-  return stage_step_payload(method, d) + (rebuilt ? 0 : d);
+  return stage_step_payload(method, d, pid) + (rebuilt ? 0 : d);
 }
-int stage_segw_of(int method, int d) { return ((3 + d + stage_step_payload(method, d)) + 1) & ~1; }
+int stage_segw_of(int method, int d, int pid) { return ((3 + d + stage_step_payload(method, d, pid)) + 1) & ~1; }
 
 // Counters that the kernels update; one small device block per record.
 struct Counters {
@@ -527,9 +528,9 @@ int auto_ckpt_k(const gs_record* r, int problem, int d, int64_t n) {
 // driver call to learn, does not matter.
 bool holds_stages(const gs_record* r, const Call& c, int64_t n, int n_save, double rtol) {
   const long long m = n > 0 ? n : 1;
-  return r->arena && r->segw == stage_segw_of(c.method, c.pi.d) &&
+  return r->arena && r->segw == stage_segw_of(c.method, c.pi.d, c.problem) &&
          r->arena_cap >= m * (step_guess(c.problem, rtol, c.method) + 1) &&
-         r->side_cap >= (size_t)m * (size_t)(n_save > 0 ? n_save : 1) * (size_t)stage_side_payload(c.method, c.pi.d);
+         r->side_cap >= (size_t)m * (size_t)(n_save > 0 ? n_save : 1) * (size_t)stage_side_payload(c.method, c.pi.d, c.problem);
 }
 
 // Stored stages when the caller allows them (gs_solve_grad), the method and
@@ -537,32 +538,39 @@ bool holds_stages(const gs_record* r, const Call& c, int64_t n, int n_save, doub
 // shared weights, a segment within MAX_STAGE_SEGW doubles), k is automatic, and
 // the expected record with its side-step stages takes at most 70% of the free
 // device memory (plus what this workspace already holds).
-bool choose_stages(const gs_record* r, const Call& c, int64_t n, int n_save, double rtol) {
+// The neural Robertson's lane-group form stores them too, in gs_solve_grad's own
+// workspace (allow_net; record handles of shared-weight problems stay compact).
+bool choose_stages(const gs_record* r, const Call& c, int64_t n, int n_save, double rtol, bool allow_net = false) {
   if (c.method != GS_METHOD_TSIT5 && c.method != GS_METHOD_RODAS5P && c.method != GS_METHOD_VERNER7 &&
       c.method != GS_METHOD_ROSENBROCK23)
     return false;
-  if (c.precision != GS_FP64 || c.pi.n_shared > 0 || c.k > 1) return false;
-  if (stage_segw_of(c.method, c.pi.d) > MAX_STAGE_SEGW) return false;
+  if (c.precision != GS_FP64 || c.k > 1) return false;
+  if (c.pi.n_shared > 0) {
+    if (!allow_net || c.problem != GS_NEURAL_ROBERTSON || c.method != GS_METHOD_RODAS5P || n > NR_GROUP_STAGES_MAX)
+      return false;
+  } else if (stage_segw_of(c.method, c.pi.d, c.problem) > MAX_STAGE_SEGW) {
+    return false;
+  }
   if (holds_stages(r, c, n, n_save, rtol)) return true;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
   const double held = (double)r->arena_cap * r->segw * sizeof(double) + (double)r->side_cap * sizeof(double);
   const double m = (double)(n > 0 ? n : 1);
   const double want =
-      m * (1.1 * step_guess(c.problem, rtol, c.method) + 1.0) * stage_segw_of(c.method, c.pi.d) * sizeof(double) +
-      m * n_save * (double)stage_side_payload(c.method, c.pi.d) * sizeof(double);
+      m * (1.1 * step_guess(c.problem, rtol, c.method) + 1.0) * stage_segw_of(c.method, c.pi.d, c.problem) * sizeof(double) +
+      m * n_save * (double)stage_side_payload(c.method, c.pi.d, c.problem) * sizeof(double);
   return want <= 0.7 * ((double)free_b + held);
 }
 
 gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double t1, const double* save_t,
-                       int n_save, double rtol, double atol, bool allow_stages = false, bool allow_packed = false) {
+                       int n_save, double rtol, double atol, bool allow_stages = false, bool own = false) {  // own: gs_solve_grad's workspace
   cudaGetDevice(&r->device);
   r->problem = c.problem;
   r->method = c.method;
   r->precision = c.precision;
   r->d = c.pi.d;
   r->P = c.pi.P;
-  r->stages = (allow_stages && choose_stages(r, c, n, n_save, rtol)) ? 1 : 0;
+  r->stages = (allow_stages && choose_stages(r, c, n, n_save, rtol, own)) ? 1 : 0;
   r->k = r->stages ? 1 : (c.k > 0 ? c.k : (c.pi.n_shared > 0 ? 1 : auto_ckpt_k(r, c.problem, c.pi.d, n)));
   if (c.pi.n_shared > 0 && !r->wpart) {
     const cudaError_t e = dev_alloc(&r->wpart, (size_t)ude_max_warps() * WPART_BYTES_PER_WARP);
@@ -582,7 +590,7 @@ gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double
   if (st != GS_OK) return st;
   if (r->stages) {
     const size_t need = (size_t)(n > 0 ? n : 1) * (size_t)(n_save > 0 ? n_save : 1) *
-                        (size_t)stage_side_payload(c.method, r->d);
+                        (size_t)stage_side_payload(c.method, r->d, c.problem);
     if (r->side_cap < need) {
       cudaFree(r->side_stg);
       r->side_stg = nullptr;
@@ -590,16 +598,16 @@ gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double
       const cudaError_t e = dev_alloc(&r->side_stg, need * sizeof(double));
       if (e != cudaSuccess) {
         r->stages = 0;  // fall back to the compact record
-        r->k = c.k > 0 ? c.k : auto_ckpt_k(r, c.problem, c.pi.d, n);
+        r->k = c.k > 0 ? c.k : (c.pi.n_shared > 0 ? 1 : auto_ckpt_k(r, c.problem, c.pi.d, n));
       } else {
         r->side_cap = need;
       }
     }
   }
   // (a packed segment's index has 32 bits: far more than the expected segments fit)
-  r->packed = allow_packed && c.precision == GS_FP32_MIXED && c.method == GS_METHOD_TSIT5 && r->k == 1 &&
+  r->packed = own && c.precision == GS_FP32_MIXED && c.method == GS_METHOD_TSIT5 && r->k == 1 &&
               packed_supports(c.problem) && (double)n * step_guess(c.problem, rtol, c.method) < 2.5e8;
-  const int segw = r->stages ? stage_segw_of(c.method, r->d) : (r->packed ? PACKED_SEGW_HOST : segw_of(r->d, r->k));
+  const int segw = r->stages ? stage_segw_of(c.method, r->d, c.problem) : (r->packed ? PACKED_SEGW_HOST : segw_of(r->d, r->k));
   if (r->segw != segw) {
     cudaFree(r->arena);
     r->arena = nullptr;
@@ -626,7 +634,7 @@ gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double
     st = ensure_arena(r, want, segw);
     if (st == GS_ERR_OOM && r->stages) {  // the stored-stage record does not fit: compact record
       r->stages = 0;
-      r->k = c.k > 0 ? c.k : auto_ckpt_k(r, c.problem, c.pi.d, n);
+      r->k = c.k > 0 ? c.k : (c.pi.n_shared > 0 ? 1 : auto_ckpt_k(r, c.problem, c.pi.d, n));
       r->segw = segw_of(r->d, r->k);
       st = ensure_arena(r, m * ((step_guess(c.problem, rtol, c.method) + r->k - 1) / r->k + 1) + slack, r->segw);
       // (the block size chosen above stays: it depends on the ensemble, not the layout)

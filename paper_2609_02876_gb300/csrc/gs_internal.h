@@ -12,6 +12,11 @@ constexpr int KMAX_HOST = 32;  // largest checkpoint interval accepted by the AB
 // Largest stored-stage segment in doubles: the record kernel stages one segment
 // per lane in shared memory (128 lanes).
 constexpr int MAX_STAGE_SEGW = 72;
+// The neural Robertson: the largest ensembles in the lane-group form (gs_nrob.cu)
+// without and with stored stages, which it alone has, and the doubles that a
+// step's stage data takes there.
+constexpr int64_t NR_GROUP_MAX = 7168, NR_GROUP_STAGES_MAX = 12288;
+constexpr int NRG_STAGE_DOUBLES = 330;
 // Arena slots the record kernel reserves per warp at a time (FwdArgs::arena_block):
 // one atomic per block instead of one per flush; at most arena_block - 1 slots
 // per warp stay unused at the end.

@@ -838,11 +838,20 @@ template <int SP>
 constexpr bool side_blocks() {
   return SP % 2 == 0;
 }
-// A (method, problem, precision) stores stages only in FP64, without shared
-// weights and when its segment fits the record kernel's staging buffer.
+// Methods that write their stage data to the segment and to the side blocks
+// themselves (store_stages / load_stages, a group's lanes together) instead of
+// staging it per lane in shared memory.
+template <class M, class = void>
+struct Direct : std::false_type {};
+template <class M>
+struct Direct<M, std::void_t<decltype(M::kDirect)>> : std::integral_constant<bool, M::kDirect> {};
+// A (method, problem, precision) stores stages only in FP64, and without shared
+// weights and when its segment fits the record kernel's staging buffer, or directly.
 template <class M, class Pb, class R>
 constexpr bool stages_possible() {
-  if constexpr (M::kStages && std::is_same<R, double>::value && !HasWeights<Pb>::value)
+  if constexpr (Direct<M>::value)
+    return true;
+  else if constexpr (M::kStages && std::is_same<R, double>::value && !HasWeights<Pb>::value)
     return stage_segw<M, Pb::D>() <= MAX_STAGE_SEGW;
   else
     return false;
@@ -1077,7 +1086,9 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
         // overwritten by the next trial if this one is rejected), so that they
         // are not held in registers across the step-size decision
         if (hard) solved = M::template trial_s<Pb, R>(xin, pin, hx, cin, yn, e, next, sd);
-        if (is_side && !group_leader<Pb>()) {
+        if constexpr (Direct<M>::value) {  // (a step's data: with its segment, below)
+          if (is_side) M::store_stages(a.side_stg + ((long long)k * ns + jp) * M::template side_payload<D>(), sd);
+        } else if (is_side && !group_leader<Pb>()) {
         } else if (is_side) {
           constexpr int SP = M::template side_payload<D>();
           if constexpr (side_blocks<SP>()) {  // this trajectory's block, 16-byte vector stores
@@ -1207,7 +1218,10 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
           const int w0 = G > 1 ? (int)(threadIdx.x & (G - 1)) : 0;
           // (unrolled for Tsit5's segments only: the longer ones of Verner7 and Rodas5P
           // raise those kernels' registers, 128 -> 162 for Verner7's Lorenz record)
-          if constexpr (STAGES && (G > 1 || std::is_same<M, Tsit5Method>::value)) {
+          if constexpr (STAGES && Direct<M>::value) {
+            if (w0 < (3 + D) / 2) dst[w0] = make_double2(stg[(2 * w0) * TB], stg[(2 * w0 + 1) * TB]);
+            M::store_stages(a.arena + idx * a.segw + 3 + D, sd);
+          } else if constexpr (STAGES && (G > 1 || std::is_same<M, Tsit5Method>::value)) {
             constexpr int SW2 = stage_segw<M, D>() / 2;
 #pragma unroll
             for (int w = 0; w < (SW2 + G - 1) / G; ++w) {
@@ -1665,7 +1679,8 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
   // unit), and there are registers to spare. (The per-lane kernels' warps hide one
   // another's loads.)
   constexpr bool AHEAD = G > 1 && !STATIC;
-  constexpr int SEGW = STAGES ? stage_segw<M, D>() : ((3 + D) + 1) & ~1;  // doubles read of a segment
+  // doubles read of a segment (direct methods read their stage data themselves)
+  constexpr int SEGW = STAGES && !Direct<M>::value ? stage_segw<M, D>() : ((3 + D) + 1) & ~1;
   double ahead[AHEAD ? SEGW : 1];
   const auto load_ahead = [&]() {
     if constexpr (AHEAD) {
@@ -1739,7 +1754,9 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
     if (k >= 0) {
       if (next_save<D, R, USER_COT>(a, s_save, k, js, tx, yx, lam, loss, us)) {
         mode = U_SIDE;  // (its length s - t is formed below, once per warp iteration)
-        if constexpr (STAGES) {
+        if constexpr (STAGES && Direct<M>::value) {
+          M::load_stages(a.side_stg + ((long long)k * ns + us) * M::template side_payload<D>(), sd);
+        } else if constexpr (STAGES) {
           constexpr int SP = M::template side_payload<D>();
           if constexpr (side_blocks<SP>()) {  // this trajectory's block, 16-byte vector loads
             const double* src = a.side_stg + ((long long)k * ns + us) * SP;
@@ -1763,6 +1780,7 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
       } else {
         // segment i: [prev, t_{i-1}, y_{i-1}[D], h_i (, Y_1..Y_5 of step i)]
         double buf[SEGW];
+        const double* sp_data = a.arena + seg * a.segw + 3 + D;
         if constexpr (AHEAD) {
 #pragma unroll
           for (int w = 0; w < SEGW; ++w) buf[w] = ahead[w];
@@ -1780,7 +1798,10 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
 #pragma unroll
         for (int c = 0; c < D; ++c) yx[c] = to_r<R>(buf[2 + c]);
         uh = buf[2 + D];
-        if constexpr (STAGES) M::template unpack<Pb, R>(false, yx, [&](int i) { return buf[3 + D + i]; }, sd);
+        if constexpr (STAGES && Direct<M>::value)
+          M::load_stages(sp_data, sd);
+        else if constexpr (STAGES)
+          M::template unpack<Pb, R>(false, yx, [&](int i) { return buf[3 + D + i]; }, sd);
         load_ahead();
         --segs_left;
         mode = U_STEP;
@@ -2021,7 +2042,8 @@ inline cudaError_t fwd_dispatch(const FwdArgs& a_in, cudaStream_t s) {
     if (e != cudaSuccess) return e;
   }
   const long long lanes = a.n * GroupOf<Pb>::value;
-  const size_t smem = (size_t)(((a.n_save + 1) & ~1) + a.segw * TPB_FWD) * sizeof(double);
+  const int staged = (Direct<M>::value && a.stages) ? ((3 + Pb::D + 1) & ~1) : a.segw;  // doubles per lane
+  const size_t smem = (size_t)(((a.n_save + 1) & ~1) + staged * TPB_FWD) * sizeof(double);
   if constexpr (SOFT) {
     const auto launch = [&](auto c64) {
       constexpr bool C64 = decltype(c64)::value;
@@ -2126,7 +2148,15 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
     if (a.k != 1) return cudaErrorInvalidValue;
     smem += weight_stage_bytes<Pb>();
     int bps = 0;
-    const auto kern = a.y_save_bar ? reverse_k1_entry<M, Pb, R, true>() : reverse_k1_entry<M, Pb, R, false>();
+    auto kern = a.y_save_bar ? reverse_k1_entry<M, Pb, R, true>() : reverse_k1_entry<M, Pb, R, false>();
+    if constexpr (stages_possible<M, Pb, R>()) {
+      if (a.stages) {
+        if (a.segw != stage_segw<M, Pb::D>()) return cudaErrorInvalidValue;
+        kern = a.y_save_bar ? reverse_k1_entry<M, Pb, R, true, true>() : reverse_k1_entry<M, Pb, R, false, true>();
+      }
+    } else {
+      if (a.stages) return cudaErrorInvalidValue;
+    }
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, TPB_REV, smem);
     cudaError_t e = persistent_launch(kern, TPB_REV, smem, lanes, s, &a);
     if (e != cudaSuccess || !a.wpart || !a.shared_w_bar) return e;

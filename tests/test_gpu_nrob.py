@@ -126,3 +126,14 @@ def test_nrob_lane_group_and_per_lane_forms(n):
         assert_close(r["y0_bar"][:, :m].cpu().numpy().T, o["y0_bar"], "y0_bar", rtol=max(1e-10, 20.0 * fy))
     wb = gs["shared_w_bar"].cpu().numpy().astype(np.float64)
     assert np.abs(wb - o["w_bar"]).max() / np.abs(o["w_bar"]).max() <= 1e-6
+    # gs_solve_grad stores every step's stages and activations up to 12288 trajectories:
+    # the group form's own bits (the same operations on the stored values)
+    info = np.zeros(2, np.int32)
+    s = api.solve_grad("nrob", Ps, Ys, wl["t0"], wl["t1"], wl["save_t"], wl["rtol"], wl["atol"], layout="soa",
+                       shared_w=SW, record_info=info)
+    assert tuple(info) == (1, 1)
+    for k in ("loss", "params_bar", "y0_bar", "shared_w_bar"):
+        assert torch.equal(s[k], gs[k]), k
+    b = api.solve_grad("nrob", P, Y, wl["t0"], wl["t1"], wl["save_t"], wl["rtol"], wl["atol"], layout="soa",
+                       shared_w=SW)
+    assert torch.equal(b["params_bar"][:, :m], s["params_bar"]) and torch.equal(b["y0_bar"][:, :m], s["y0_bar"])

@@ -130,6 +130,8 @@ struct gs_record {
   int32_t* natt = nullptr;
   int32_t* status = nullptr;
   double* y_final = nullptr;
+  int32_t* order = nullptr;  // scratch of the sweep's step-count sort (workspaces, ensembles up to ORDER_MAX)
+  int64_t order_cap = 0;
   void* wpart = nullptr;  // per-warp shared-weight gradient partials (shared-weight problems)
   // Stored stages (gs_solve_grad's workspace, Tsit5 FP64, k = 1): segments also
   // hold each step's stage data, side_stg (n x n_save x payload) the side steps'.
@@ -186,6 +188,9 @@ void free_arrays(gs_record* r) {
   cudaFree(r->natt);
   cudaFree(r->status);
   cudaFree(r->y_final);
+  cudaFree(r->order);
+  r->order = nullptr;
+  r->order_cap = 0;
   r->head = nullptr;
   r->S = r->natt = r->status = nullptr;
   r->y_final = nullptr;
@@ -197,6 +202,7 @@ constexpr int kMaxDim = 8;  // largest state dimension of the registry
 size_t record_bytes(const gs_record* r) {
   return (size_t)r->arena_cap * r->segw * sizeof(double) + r->side_cap * sizeof(double) +
          (size_t)r->n_cap * (sizeof(long long) + 3 * sizeof(int32_t) + kMaxDim * sizeof(double)) +
+         (r->order ? (ORDER_WORDS + (size_t)r->order_cap) * sizeof(int32_t) : 0) +
          sizeof(Counters);
 }
 
@@ -588,6 +594,17 @@ gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double
   if (c.kernel_ms && (st = ensure_events(r)) != GS_OK) return st;
   st = ensure_arrays(r, n, r->d);
   if (st != GS_OK) return st;
+  if (own && c.precision == GS_FP64 && c.pi.n_shared == 0 && n <= ORDER_MAX && r->order_cap < n) {
+    cudaFree(r->order);
+    r->order = nullptr;
+    r->order_cap = 0;
+    if (dev_alloc(&r->order, (ORDER_WORDS + n) * sizeof(int32_t)) == cudaSuccess) {
+      r->order_cap = n;
+    } else {  // no room: the sweep takes the trajectories as they come
+      r->order = nullptr;
+      cudaGetLastError();
+    }
+  }
   if (r->stages) {
     const size_t need = (size_t)(n > 0 ? n : 1) * (size_t)(n_save > 0 ? n_save : 1) *
                         (size_t)stage_side_payload(c.method, r->d, c.problem);
@@ -668,6 +685,7 @@ gs_status launch_reverse(const gs_record* r, const double* params, const float* 
   a.S = r->S;
   a.y_final = r->y_final;
   a.wpart = r->wpart;
+  a.order_buf = r->order_cap >= r->n ? r->order : nullptr;  // (workspaces: a handle may be swept on several streams)
   a.work = &r->ctr->work_rev;
   a.k = r->k;
   a.segw = r->segw;

@@ -94,8 +94,14 @@ struct RevArgs {
   int* tc_error;             // set when a tensor-core product's completion wait ran out (or nullptr)
   int t1_pre;                // set by the launcher: y0_bar (and loss) hold lambda (and the loss) after
                              // the save at t1, which the reverse sweep then starts from
+  int32_t* order_buf;        // scratch of the step-count sort, ORDER_WORDS + n words, or nullptr (no sort)
+  const int32_t* order;      // set by the launcher: trajectory of each ticket, or nullptr (the ticket itself)
   double save_t[MAX_SAVE_HOST];
 };
+// Largest ensemble whose reverse sweep is sorted by step count (measured to here; the
+// order is 64 MB then), and the sort's scratch besides the order itself.
+constexpr int64_t ORDER_MAX = 1 << 24;
+constexpr int ORDER_WORDS = 1024;
 
 // Arguments of the forward-mode (tangent) replay kernels. Direction q of a
 // launch is direction dir0 + q of the call.

@@ -1708,7 +1708,7 @@ __device__ __forceinline__ void reverse_k1_body(const RevArgs& a) {
       }
       if (need) {
         if (got < n) {
-          k = got;
+          k = a.order ? a.order[got] : got;
           const long long hd = a.head[k];
           if (a.status[k] != TRAJ_OK || hd < 0) {
             if (group_leader<Pb>()) write_nan<NP, D>(a, k);
@@ -1974,7 +1974,8 @@ inline int sm_count() {
 // ensemble needs).
 template <class Kern>
 inline cudaError_t persistent_launch(Kern kern, int tpb, size_t smem, long long n, cudaStream_t s,
-                                     const void* args_ptr) {  // n: lanes with work
+                                     const void* args_ptr, int max_ctas = 1 << 20) {
+  // n: lanes with work; max_ctas: most CTAs per SM
   cudaError_t err = cudaSuccess;
   if (smem > 32 * 1024)  // (static and dynamic together have 48 KB without it)
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1985,6 +1986,7 @@ inline cudaError_t persistent_launch(Kern kern, int tpb, size_t smem, long long 
     int bps = 0;
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, tpb, smem);
     if (err != cudaSuccess) return err;
+    if (bps > max_ctas) bps = max_ctas;
     blocks *= bps > 0 ? bps : 1;
   }
   if (blocks > need) blocks = need;
@@ -2137,6 +2139,73 @@ inline bool t1_save_pass(const RevArgs& a, cudaStream_t s, cudaError_t* err) {
   }
 }
 
+// Trajectories by decreasing step count, for the sweep's tickets (a counting sort;
+// equal counts in any order). A warp costs its FP64 unit what its longest lanes cost,
+// and an FP64 instruction takes as long for one lane as for 32: sorted, the lanes of a
+// warp end together, and the shortest trajectories come last and even out the units'
+// ends. Sweeps without / with it, ms: Van der Pol 65521 2.29 / 2.16, 98304 3.63 / 2.90,
+// 2^20 24.6 / 23.8; Lorenz 26000 0.666 / 0.622, 98304 1.91 / 1.54, 2^24 225 / 218;
+// Robertson 2^18 31.5 / 29.0; HIRES 50000 72.2 / 52.0. The FP32-mixed sweeps are bound by
+// their segments' reads, which the order scatters (Lorenz 2^20 1.22 / 1.27): not sorted.
+constexpr int ORDER_BINS = ORDER_WORDS;
+constexpr int ORDER_TPB = 256;
+__device__ __forceinline__ int order_bin(int s) { return s < 0 ? 0 : (s < ORDER_BINS ? s : ORDER_BINS - 1); }
+static __global__ void __launch_bounds__(ORDER_TPB) order_count_kernel(const int32_t* S, int n, int32_t* bins) {
+  __shared__ int32_t cnt[ORDER_BINS];
+  for (int i = threadIdx.x; i < ORDER_BINS; i += ORDER_TPB) cnt[i] = 0;
+  __syncthreads();
+  const int k = blockIdx.x * ORDER_TPB + threadIdx.x;
+  if (k < n) atomicAdd(&cnt[order_bin(S[k])], 1);
+  __syncthreads();
+  for (int i = threadIdx.x; i < ORDER_BINS; i += ORDER_TPB)
+    if (cnt[i]) atomicAdd(&bins[i], cnt[i]);
+}
+// bins[b] becomes the number of trajectories in the bins above b (one block).
+static __global__ void __launch_bounds__(ORDER_BINS) order_scan_kernel(int32_t* bins) {
+  __shared__ int32_t sum[ORDER_BINS];
+  const int i = threadIdx.x, b = ORDER_BINS - 1 - i;  // descending
+  const int32_t own = bins[b];
+  sum[i] = own;
+  __syncthreads();
+  for (int d = 1; d < ORDER_BINS; d <<= 1) {
+    const int32_t v = i >= d ? sum[i - d] : 0;
+    __syncthreads();
+    sum[i] += v;
+    __syncthreads();
+  }
+  bins[b] = sum[i] - own;
+}
+// A block takes its share of each bin with one atomic.
+static __global__ void __launch_bounds__(ORDER_TPB) order_place_kernel(const int32_t* S, int n, int32_t* bins,
+                                                                      int32_t* order) {
+  __shared__ int32_t cnt[ORDER_BINS], base[ORDER_BINS];
+  for (int i = threadIdx.x; i < ORDER_BINS; i += ORDER_TPB) cnt[i] = 0;
+  __syncthreads();
+  const int k = blockIdx.x * ORDER_TPB + threadIdx.x;
+  const int b = k < n ? order_bin(S[k]) : 0;
+  const int rank = k < n ? atomicAdd(&cnt[b], 1) : 0;
+  __syncthreads();
+  for (int i = threadIdx.x; i < ORDER_BINS; i += ORDER_TPB)
+    if (cnt[i]) base[i] = atomicAdd(&bins[i], cnt[i]);
+  __syncthreads();
+  if (k < n) order[base[b] + rank] = k;
+}
+// Sorts into a.order_buf ([ORDER_BINS] bins, then [n]) when the launch is of that
+// kind: more than one warp per FP64 unit (with one, the longest trajectory decides).
+inline cudaError_t order_pass(RevArgs& a, cudaStream_t s) {
+  a.order = nullptr;
+  const long long unit = (long long)sm_count() * 4 * 32;
+  if (!a.order_buf || a.n <= unit || a.n > ORDER_MAX) return cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(a.order_buf, 0, ORDER_BINS * sizeof(int32_t), s);
+  if (e != cudaSuccess) return e;
+  const unsigned blocks = (unsigned)((a.n + ORDER_TPB - 1) / ORDER_TPB);
+  order_count_kernel<<<blocks, ORDER_TPB, 0, s>>>(a.S, (int)a.n, a.order_buf);
+  order_scan_kernel<<<1, ORDER_BINS, 0, s>>>(a.order_buf);
+  order_place_kernel<<<blocks, ORDER_TPB, 0, s>>>(a.S, (int)a.n, a.order_buf, a.order_buf + ORDER_BINS);
+  a.order = a.order_buf + ORDER_BINS;
+  return cudaGetLastError();
+}
+
 template <class M, class Pb, class R, bool SOFT = false>
 inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
   RevArgs a = a_in;
@@ -2173,6 +2242,9 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
     cudaError_t e;
     a.t1_pre = t1_save_pass<Pb, R>(a, s, &e) ? 1 : 0;
     if (e != cudaSuccess) return e;
+    if constexpr (std::is_same<R, double>::value) {
+      if ((e = order_pass(a, s)) != cudaSuccess) return e;
+    }
   }
   if constexpr (SOFT) {
     if constexpr (stages_possible<M, Pb, R>()) {
@@ -2200,8 +2272,16 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
     if (a.stages) return cudaErrorInvalidValue;
   }
   if (a.k == 1) {
-    if (a.y_save_bar) return persistent_launch(reverse_k1_entry<M, Pb, R, true>(), TPB_REV, smem, lanes, s, &a);
-    return persistent_launch(reverse_k1_entry<M, Pb, R, false>(), TPB_REV, smem, lanes, s, &a);
+    // A sorted sweep of a large step (HIRES with Rodas5P) runs one CTA per SM: a warp
+    // alone keeps its FP64 unit 85% busy (two 95%), and with a trajectory per lane at
+    // a time the tickets, longest first, even out the units' ends: up to two waves of
+    // such CTAs. HIRES sweeps with 2 / 1 CTAs per SM: 20000 39.3 / 23.3, 30000 40.1 / 36.1,
+    // 38912 41.4 / 39.4, 65536 66.6 / 69.5 ms.
+    const bool alone = a.order && std::is_same<M, Rodas5PMethod>::value && Pb::D > 3 &&
+                       a.n <= 2ll * sm_count() * TPB_REV;
+    const int ctas = alone ? 1 : 1 << 20;
+    if (a.y_save_bar) return persistent_launch(reverse_k1_entry<M, Pb, R, true>(), TPB_REV, smem, lanes, s, &a, ctas);
+    return persistent_launch(reverse_k1_entry<M, Pb, R, false>(), TPB_REV, smem, lanes, s, &a, ctas);
   }
   if constexpr (GroupOf<Pb>::value > 1) {
     return cudaErrorInvalidValue;  // (lane groups sweep k = 1 records)

@@ -621,9 +621,11 @@ gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double
       }
     }
   }
-  // (a packed segment's index has 32 bits: far more than the expected segments fit)
+  // A packed segment's index has 31 bits; with more segments than expected the rerun is
+  // in the general layout. Van der Pol 3000001 / 2^22 trajectories, general / packed ms:
+  // 14.3 / 9.0, 19.8 / 12.4.
   r->packed = own && c.precision == GS_FP32_MIXED && c.method == GS_METHOD_TSIT5 && r->k == 1 &&
-              packed_supports(c.problem) && (double)n * step_guess(c.problem, rtol, c.method) < 2.5e8;
+              packed_supports(c.problem) && (double)n * step_guess(c.problem, rtol, c.method) < 1.5e9;
   const int segw = r->stages ? stage_segw_of(c.method, r->d, c.problem) : (r->packed ? PACKED_SEGW_HOST : segw_of(r->d, r->k));
   if (r->segw != segw) {
     cudaFree(r->arena);
@@ -827,10 +829,10 @@ gs_status solve_grad_in(gs_record* r, const Call& c, int64_t n, const double* pa
 
 // An FP32-mixed gs_solve_grad of more than two chunks runs chunk by chunk
 // (shared-weight problems, step_counts and a wait deadline excepted): the
-// compact record of 2^21 Lorenz trajectories takes ~5.5 GB against ~44 GB at
-// 2^24, and the reverse sweep's scattered per-lane segment reads run faster
-// over the smaller arena (Lorenz 2^24, rtol 1e-6, measured: 48.7 / 43.3 / 40.7
-// / 40.4 / 41.4 ms in chunks of 2^18 / 2^19 / 2^20 / 2^21 / 2^22 against 44.0
+// record of 2^21 Lorenz trajectories takes ~3.4 GB against ~27 GB at 2^24, and the
+// reverse sweep's scattered per-lane segment reads run faster over the smaller
+// arena (Lorenz 2^24, rtol 1e-6, measured: 26.7 / 26.2 / 26.0 ms in chunks of 2^20 /
+// 2^21 / 2^22; with the general segments 40.7 / 40.4 / 41.4 against 44.0
 // ms in one piece). Trajectories are independent, so
 // the results equal the one-piece call bit for bit.
 //

@@ -48,6 +48,24 @@ def test_spans_and_save_grids(t0, t1, saves):
     both("lorenz", wl["params"], wl["y0"], t0, t1, saves, 1e-5, 1e-7)
 
 
+@pytest.mark.parametrize("n,rtol", [(3000001, 1e-6), (1 << 22, 1e-8)])
+def test_large_ensembles_in_one_piece(n, rtol):
+    """Up to the largest one-piece call and some 1e9 segments: parts solved alone have the same bits."""
+    build.build()
+    wl = W.make("vdp", n, rtol=rtol)
+    P, Y = dev(wl["params"].T), dev(wl["y0"].T)
+
+    def grad(lo, hi):
+        return api.solve_grad("vdp", P[:, lo:hi].contiguous(), Y[:, lo:hi].contiguous(), wl["t0"], wl["t1"],
+                              wl["save_t"], wl["rtol"], wl["atol"], layout="soa", precision="fp32_mixed")
+
+    g = grad(0, n)
+    for lo in (0, n // 2, n - 3000):
+        part = grad(lo, lo + 3000)
+        for k in ("loss", "params_bar", "y0_bar", "status"):
+            assert torch.equal(g[k][..., lo:lo + 3000], part[k]), k
+
+
 @pytest.mark.parametrize("kw", [dict(max_steps=20), dict(h0=1e-3), dict(h0=10.0)])
 def test_options_and_failed_trajectories(kw):
     n = 777

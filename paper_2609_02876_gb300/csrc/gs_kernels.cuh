@@ -2089,14 +2089,27 @@ inline cudaError_t fwd_dispatch(const FwdArgs& a_in, cudaStream_t s) {
           return persistent_launch(record_kernel_mb<M, Pb, R, true, true, false, 3>, TPB_FWD, smem, lanes, s, &a);
         return persistent_launch(record_kernel_mb<M, Pb, R, true, true, false, 1>, TPB_FWD, smem, lanes, s, &a);
       } else {
-        return persistent_launch(record_kernel<M, Pb, R, true, true>, TPB_FWD, smem, lanes, s, &a);
+        // Rosenbrock23 (Robertson: 148 registers, 3 CTAs per SM): two waves of 2 CTAs where 3
+        // leave a short second wave. Robertson record of 65536 with 3 / 2: 22.1 / 15.3 ms.
+        const long long wave = (long long)sm_count() * TPB_FWD;
+        const bool two =
+            std::is_same<M, Ros23Method>::value && Pb::D == 3 && lanes > 3 * wave && lanes <= 4 * wave;
+        return persistent_launch(record_kernel<M, Pb, R, true, true>, TPB_FWD, smem, lanes, s, &a, two ? 2 : 1 << 20);
       }
     }
   } else {
     if (a.stages) return cudaErrorInvalidValue;
   }
-  if (a.y_save) return persistent_launch(record_kernel<M, Pb, R, true, false>, TPB_FWD, smem, lanes, s, &a);
-  return persistent_launch(record_kernel<M, Pb, R, false, false>, TPB_FWD, smem, lanes, s, &a);
+  int ctas = 1 << 20;
+  if constexpr (std::is_same<M, Rodas5PMethod>::value && std::is_same<Pb, NeuralRobertson>::value) {
+    // 3 CTAs per SM fit, and a warp keeps its FP64 unit busy, so a CTA more only costs
+    // where it does not save a wave: records of 65536 trajectories 307 ms with 2 and 438 with
+    // 3, of 56000 220 ms with 3.
+    const long long wave = (long long)sm_count() * TPB_FWD;
+    if (3 * ((lanes + 3 * wave - 1) / (3 * wave)) >= 2 * ((lanes + 2 * wave - 1) / (2 * wave))) ctas = 2;
+  }
+  if (a.y_save) return persistent_launch(record_kernel<M, Pb, R, true, false>, TPB_FWD, smem, lanes, s, &a, ctas);
+  return persistent_launch(record_kernel<M, Pb, R, false, false>, TPB_FWD, smem, lanes, s, &a, ctas);
   }
 }
 

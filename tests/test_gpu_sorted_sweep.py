@@ -35,3 +35,25 @@ def test_same_as_unsorted(problem, n, span, fail):
     for k in ("loss", "params_bar", "y0_bar"):
         a, b = g[k].nan_to_num(7.0), r[k].nan_to_num(7.0)
         assert torch.equal(a, b), k
+
+
+@pytest.mark.parametrize("problem,method,n", [("robertson", "rosenbrock23", 58369), ("nrob", None, 58368),
+                                              ("nrob", None, 58369)])
+def test_records_at_the_edge_of_three_waves(problem, method, n):
+    """Where the record changes its CTAs per SM (58368 = 3 x 152 x 128 lanes): the last
+    trajectories have the bits that they have among a few."""
+    build.build()
+    wl = W.make(problem, n)
+    P, Y = dev(wl["params"].T), dev(wl["y0"].T)
+    kw = dict(layout="soa", method=method)
+    if wl["w"] is not None:
+        kw["shared_w"] = torch.as_tensor(np.asarray(wl["w"], np.float32), device="cuda")
+
+    def final(lo):
+        p, y = P[:, lo:].contiguous(), Y[:, lo:].contiguous()
+        args = (problem, p, y, wl["t0"], wl["t1"], wl["save_t"], wl["rtol"], wl["atol"])
+        if method:
+            return api.solve_grad(*args, **kw)["params_bar"]
+        return api.solve(*args, want_saves=False, **kw)["y_final"]
+
+    assert torch.equal(final(0)[:, n - 30000:], final(n - 30000))

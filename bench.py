@@ -69,15 +69,14 @@ STIFF = {"robertson", "hires", "nrob"}
 
 
 # DRAM bytes per accepted step, read + write, measured with ncu (dram__bytes_read.sum +
-# dram__bytes_write.sum, one launch of each kernel) on the first 2^20 trajectories of
-# the same FP64 workload, stored-stage layout (Lorenz: 45.15 accepted steps per
-# trajectory; Robertson: 101243901 accepted steps in all); a launch's traffic grows
-# in proportion to its accepted steps. The Lorenz reverse sweep's writes are its
-# register spills (the kernel is capped at 96 registers).
-TRAFFIC_PER_STEP = {("lorenz", "fp64", "reverse", "stages"): (14935465472 + 328079616) / (45.15 * 2 ** 20),
-                    ("lorenz", "fp64", "record", "stages"): (291875328 + 9850115584) / (45.15 * 2 ** 20),
-                    ("robertson", "fp64", "reverse", "stages"): (49664537600 + 67086336) / 101243901,
-                    ("robertson", "fp64", "record", "stages"): (2908891648 + 67400810240) / 101243901}
+# dram__bytes_write.sum, one launch of each kernel) on the same FP64 workload,
+# stored-stage layout (Lorenz: 2^20 trajectories, 47348406 accepted steps in
+# all; Robertson: 2^18 trajectories, 25311560); a launch's traffic grows in
+# proportion to its accepted steps.
+TRAFFIC_PER_STEP = {("lorenz", "fp64", "reverse", "stages"): (16558314240 + 202626560) / 47348406,
+                    ("lorenz", "fp64", "record", "stages"): (266159872 + 9855549184) / 47348406,
+                    ("robertson", "fp64", "reverse", "stages"): (18115212288 + 41250304) / 25311560,
+                    ("robertson", "fp64", "record", "stages"): (471803648 + 12487128576) / 25311560}
 
 # Nominal FMA lanes per SM per clock of this part (FP64 at 1/64 of FP32), for the
 # nominal peak printed beside the measured one.
@@ -557,13 +556,16 @@ def forward_measure(args, peaks, steps=5):
 
 def launches_per_step(problem, precision, k, wl):
     """Kernels one gs_solve_grad call launches: the starting-step pass, the record, the
-    t1-save pass (FP64, no shared weights, k = 1, last save time t1), the reverse sweep,
-    and for shared-weight problems the weight-gradient reduction."""
+    t1-save pass (FP64, no shared weights, k = 1, last save time t1), the sort of the
+    trajectories by step count (three kernels; FP64, no shared weights, more trajectories
+    than one warp per FP64 unit and up to 2^24), the reverse sweep, and for shared-weight
+    problems the weight-gradient reduction."""
     weights = problem in ("lv_ude", "nrob")
     st = np.asarray(wl["save_t"], dtype=np.float64)
     t1_pass = (precision == "fp64" and not weights and k == 1 and st.size > 0
                and st[-1].tobytes() == np.float64(wl["t1"]).tobytes())
-    return 3 + int(t1_pass) + int(weights)
+    sort = precision == "fp64" and not weights and 152 * 4 * 32 < len(wl["y0"]) <= 1 << 24
+    return 3 + int(t1_pass) + 3 * int(sort) + int(weights)
 
 
 def record_memory_measure():

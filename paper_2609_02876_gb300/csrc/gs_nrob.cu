@@ -8,15 +8,13 @@ namespace gs {
 // besides its stage data, the network's activations at the eight stages, so the
 // reverse sweep evaluates no network at all (a unit spent 116000 of its 209000
 // cycles on the step's recompute). The lanes of a group write and read their own
-// neurons' activations, whole 128-byte lines; the leader writes the rest.
+// neurons' activations, 128 bytes in a row each time (from any 16-byte boundary);
+// the leader writes the rest.
 struct NrGroupMethod : Rodas5PMethod {
   using G = NeuralRobertsonGroup;
   static constexpr bool kDirect = true;
-  static constexpr int D = 3, ACT = 2 * NR_H * 8;  // activations of a step
-  struct Data {
-    double z3[8], Y[8][D], U[8][D], LU[D][D], rinv[D], ynew[D], piv[D];
-  };
-  static_assert(ACT + sizeof(Data) / sizeof(double) == NRG_STAGE_DOUBLES && NRG_STAGE_DOUBLES % 2 == 0, "layout");
+  static constexpr int D = 3, ACT = G::ACT;
+  using Data = G::Data;
   template <class Pb, class R>
   struct StageData {
     Data d;

@@ -20,6 +20,7 @@
 #pragma once
 
 #include "gs_device.cuh"
+#include "gs_internal.h"
 
 namespace gs {
 
@@ -444,6 +445,15 @@ struct NeuralRobertsonGroup {
     Fwd F[8];
     double sg[8];  // sigmoid(z3) of each stage (the reverse of the step)
   };
+  // Stored stages: what a step's data holds besides the activations of its eight
+  // stages, the same on every lane of the group. Read and written as double2, so
+  // aligned to 16 bytes wherever the compiler keeps it (registers or local memory).
+  static constexpr int ACT = 2 * NR_H * 8;  // activations of a step
+  struct alignas(16) Data {
+    double z3[8], Y[8][D], U[8][D], LU[D][D], rinv[D], ynew[D], piv[D];
+  };
+  static_assert(alignof(Data) == sizeof(double2) && ACT % 2 == 0, "double2 accesses");
+  static_assert(ACT + sizeof(Data) / sizeof(double) == NRG_STAGE_DOUBLES && NRG_STAGE_DOUBLES % 2 == 0, "layout");
   __device__ __forceinline__ static void forward(const double (&x)[D], Fwd& F) {
     asm volatile("" ::: "memory");  // (the weights are re-read at every use, as in the per-lane form)
     const double* w = weights();

@@ -117,7 +117,7 @@ struct gs_record {
   int device = 0;
   int problem = 0, method = GS_METHOD_TSIT5, precision = GS_FP64;
   int d = 0, P = 0, k = 0, segw = 0;
-  int arena_block = 32;  // arena slots the record kernel reserves per warp at a time
+  int arena_block = 32;  // arena slots the record kernel reserves per 32 trajectories at a time
   int64_t n = 0;
   double t0 = 0, t1 = 0, rtol = 0, atol = 0;
   int n_save = 0;
@@ -633,9 +633,10 @@ gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double
     r->arena_cap = 0;
     r->segw = segw;
   }
-  // Expected segments, plus the unused tails of the record kernel's per-warp slot
-  // blocks: a warp reserves about an eighth of its expected segments at a time
-  // (32 to ARENA_BLOCK_HOST slots), and leaves less than one block unused.
+  // Expected segments, plus the unused tails of the record kernel's slot blocks: 32
+  // trajectories (one warp, or the warps of their lane groups) reserve about an eighth
+  // of their expected segments at a time (32 to ARENA_BLOCK_HOST slots), and leave less
+  // than that unused.
   const long long m = n > 0 ? n : 1;
   const long long per_traj = (step_guess(c.problem, rtol, c.method) + r->k - 1) / r->k + 1;
   const long long warps = std::min<long long>((m + 31) / 32, 4096 * 4);

@@ -17,9 +17,10 @@ constexpr int MAX_STAGE_SEGW = 72;
 // step's stage data takes there.
 constexpr int64_t NR_GROUP_MAX = 7168, NR_GROUP_STAGES_MAX = 12288;
 constexpr int NRG_STAGE_DOUBLES = 330;
-// Arena slots the record kernel reserves per warp at a time (FwdArgs::arena_block):
-// one atomic per block instead of one per flush; at most arena_block - 1 slots
-// per warp stay unused at the end.
+// Arena slots the record kernel reserves at a time per 32 trajectories
+// (FwdArgs::arena_block; a warp with G lanes per trajectory reserves 1/G of it): one
+// atomic per block instead of one per flush; less than a block per 32 trajectories
+// stays unused at the end.
 constexpr int ARENA_BLOCK_HOST = 256;
 
 // Doubles per compact record segment [prev, t_start, y_start[d], h[k]], rounded
@@ -52,7 +53,7 @@ struct FwdArgs {
   int* any_failed;                // set when a trajectory ends with a non-OK status
   int k;                          // accepted steps per segment
   int segw;                       // doubles per segment
-  int arena_block;                // slots a warp reserves at a time (>= 32; 0 means ARENA_BLOCK_HOST)
+  int arena_block;                // slots reserved at a time per 32 trajectories (>= 32; 0 means ARENA_BLOCK_HOST)
   // Stored stages (k = 1, FP64): each segment also holds its step's stage
   // data after h (Tsit5: Y_1..Y_5; Verner7: Y_1..Y_8; Rodas5P: U_0..U_7 and
   // the LU of W with pivot reciprocals and pivots; Rosenbrock23: k1, u2 and the

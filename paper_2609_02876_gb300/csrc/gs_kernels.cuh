@@ -1192,10 +1192,11 @@ __device__ __forceinline__ void record_body(const FwdArgs& a) {
     if (__any_sync(FULL_MASK, flush)) {
       // arena slots are reserved per warp in blocks (one atomic per block, not
       // per flush); the unused tail of a warp's last block stays empty, since
-      // segments are linked, not indexed
+      // segments are linked, not indexed. A lane group's warp carries fewer trajectories
+      // and reserves as much less: 32 trajectories leave the same tail in every form.
       const unsigned fm = __ballot_sync(FULL_MASK, flush && group_leader<Pb>());
       const int cnt = __popc(fm), rem = (int)(res_end - res_next);
-      const int blk = a.arena_block >= 32 ? a.arena_block : ARENA_BLOCK_HOST;
+      const int blk = (a.arena_block >= 32 ? a.arena_block : ARENA_BLOCK_HOST) / GroupOf<Pb>::value;
       long long nb = 0;
       if (cnt > rem) {  // warp-uniform: a new block continues where the reserved one ends
         unsigned long long base = 0;

@@ -514,13 +514,24 @@ gs_status run_record(gs_record* r, const Call& c, int64_t n, const double* param
   return GS_ERR_OOM;
 }
 
+// Whether a call with k = 1 records packed segments (own: gs_solve_grad's workspace).
+// A packed segment's index has 31 bits; with more segments than expected the rerun is
+// in the general layout. Van der Pol 3000001 / 2^22 trajectories, general / packed ms:
+// 14.3 / 9.0, 19.8 / 12.4.
+bool packed_call(const Call& c, int64_t n, double rtol, bool own) {
+  return own && c.precision == GS_FP32_MIXED && c.method == GS_METHOD_TSIT5 && packed_supports(c.problem) &&
+         (double)n * step_guess(c.problem, rtol, c.method) < 1.5e9;
+}
+
 // Checkpoint interval when the caller leaves it to the library: k = 1 (every
 // accepted state stored, nothing recomputed in the reverse sweep) if the
 // expected record takes at most half of the free device memory, else a
 // 128-byte segment of 14 - d steps (one checkpoint per 14 - d steps).
-int auto_ckpt_k(const gs_record* r, int problem, int d, int64_t n) {
-  if (r->arena && (r->segw == segw_of(d, 1) || r->packed) && r->arena_cap >= (n > 0 ? n : 1) * (long long)(step_guess(problem) + 1))
-    return 1;  // held from an earlier call of this size
+int auto_ckpt_k(const gs_record* r, const Call& c, int64_t n, double rtol, bool own) {
+  const int problem = c.problem, d = c.pi.d;
+  const int segw = packed_call(c, n, rtol, own) ? PACKED_SEGW_HOST : segw_of(d, 1);
+  if (r->arena && r->segw == segw && r->arena_cap >= (n > 0 ? n : 1) * (long long)(step_guess(problem) + 1))
+    return 1;  // held from an earlier call of this size, in this call's layout
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = 0;
   const size_t held = (size_t)r->arena_cap * r->segw * sizeof(double);  // reusable by this record
@@ -577,7 +588,7 @@ gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double
   r->d = c.pi.d;
   r->P = c.pi.P;
   r->stages = (allow_stages && choose_stages(r, c, n, n_save, rtol, own)) ? 1 : 0;
-  r->k = r->stages ? 1 : (c.k > 0 ? c.k : (c.pi.n_shared > 0 ? 1 : auto_ckpt_k(r, c.problem, c.pi.d, n)));
+  r->k = r->stages ? 1 : (c.k > 0 ? c.k : (c.pi.n_shared > 0 ? 1 : auto_ckpt_k(r, c, n, rtol, own)));
   if (c.pi.n_shared > 0 && !r->wpart) {
     const cudaError_t e = dev_alloc(&r->wpart, (size_t)ude_max_warps() * WPART_BYTES_PER_WARP);
     if (e != cudaSuccess) return cuda_fail(e);
@@ -615,17 +626,13 @@ gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double
       const cudaError_t e = dev_alloc(&r->side_stg, need * sizeof(double));
       if (e != cudaSuccess) {
         r->stages = 0;  // fall back to the compact record
-        r->k = c.k > 0 ? c.k : (c.pi.n_shared > 0 ? 1 : auto_ckpt_k(r, c.problem, c.pi.d, n));
+        r->k = c.k > 0 ? c.k : (c.pi.n_shared > 0 ? 1 : auto_ckpt_k(r, c, n, rtol, own));
       } else {
         r->side_cap = need;
       }
     }
   }
-  // A packed segment's index has 31 bits; with more segments than expected the rerun is
-  // in the general layout. Van der Pol 3000001 / 2^22 trajectories, general / packed ms:
-  // 14.3 / 9.0, 19.8 / 12.4.
-  r->packed = own && c.precision == GS_FP32_MIXED && c.method == GS_METHOD_TSIT5 && r->k == 1 &&
-              packed_supports(c.problem) && (double)n * step_guess(c.problem, rtol, c.method) < 1.5e9;
+  r->packed = r->k == 1 && packed_call(c, n, rtol, own);
   const int segw = r->stages ? stage_segw_of(c.method, r->d, c.problem) : (r->packed ? PACKED_SEGW_HOST : segw_of(r->d, r->k));
   if (r->segw != segw) {
     cudaFree(r->arena);
@@ -654,7 +661,7 @@ gs_status setup_record(gs_record* r, const Call& c, int64_t n, double t0, double
     st = ensure_arena(r, want, segw);
     if (st == GS_ERR_OOM && r->stages) {  // the stored-stage record does not fit: compact record
       r->stages = 0;
-      r->k = c.k > 0 ? c.k : (c.pi.n_shared > 0 ? 1 : auto_ckpt_k(r, c.problem, c.pi.d, n));
+      r->k = c.k > 0 ? c.k : (c.pi.n_shared > 0 ? 1 : auto_ckpt_k(r, c, n, rtol, own));
       r->segw = segw_of(r->d, r->k);
       st = ensure_arena(r, m * ((step_guess(c.problem, rtol, c.method) + r->k - 1) / r->k + 1) + slack, r->segw);
       // (the block size chosen above stays: it depends on the ensemble, not the layout)

@@ -265,10 +265,13 @@ void destroy(gs_record* r) {
   delete r;
 }
 
-// Freed records of at most POOL_RECORD_BYTES, kept for the next
-// gs_forward_record of the same call signature (a training loop records and
-// frees one per step; allocating and freeing its buffers took 0.45 ms of a 2.0 ms
-// step at 10007 Lorenz trajectories). At most POOL_RECORDS of them; the oldest is
+// Freed records of at most POOL_RECORD_BYTES, the shared-weight problems' partials
+// included, kept for the next gs_forward_record of the same call signature (a
+// training loop records and frees one per step; allocating and freeing its buffers
+// took 0.45 ms of a 2.0 ms step at 10007 Lorenz trajectories). The limits bound what
+// the library holds beside the caller's allocator, 256 MB in all; with 10 saves a
+// Lorenz record stays below them up to about 12300 trajectories, with 50 saves a Van
+// der Pol record up to about 7100. At most POOL_RECORDS of them; the oldest is
 // released for a newer one, and all of them when an allocation fails. A record
 // enters the pool after the device has finished all work, as cudaFree would have
 // waited for, so any stream may use it next.
@@ -292,7 +295,9 @@ gs_record* pool_take(const RecordKey& key) {
 }
 
 bool pool_put(gs_record* r) {  // false: the caller releases it
-  if (!r || !r->arena || record_bytes(r) > POOL_RECORD_BYTES) return false;
+  if (!r || !r->arena) return false;
+  const size_t partials = r->wpart ? (size_t)ude_max_warps() * WPART_BYTES_PER_WARP : 0;
+  if (record_bytes(r) + partials > POOL_RECORD_BYTES) return false;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev != r->device) return false;
   if (cudaDeviceSynchronize() != cudaSuccess) return false;

@@ -1,5 +1,5 @@
 """What a call chooses by the device memory that is free, with most of it taken,
-and what it keeps."""
+and what the pool of freed records keeps."""
 import numpy as np
 import pytest
 import torch
@@ -52,3 +52,20 @@ def test_interval_after_a_packed_solve_follows_the_free_memory():
         hogs.clear()
         ctx.close()
         torch.cuda.empty_cache()
+
+
+def test_pool_counts_the_weight_partials():
+    """A neural Robertson record of 111 MiB has 26 MiB of weight-gradient partials
+    besides: together more than the pool keeps, so freeing it gives all back."""
+    wl = W.make("nrob", 9101)
+    w = torch.as_tensor(np.asarray(wl["w"], dtype=np.float32), device="cuda")
+    P, Y = dev(wl["params"].T), dev(wl["y0"].T)
+    used = []
+    for n in (9100, 9101):  # (the first also loads the kernels)
+        Pn, Yn = P[:, :n].contiguous(), Y[:, :n].contiguous()
+        free = torch.cuda.mem_get_info()[0]
+        rec, _, _ = api.forward_record("nrob", Pn, Yn, *args(wl), layout="soa", shared_w=w, want_saves=False)
+        assert (100 << 20) < rec.bytes() < (128 << 20)
+        rec.free()
+        used.append(free - torch.cuda.mem_get_info()[0])
+    assert used[1] < (16 << 20), used

@@ -146,6 +146,14 @@ cudaError_t launch_fwd_index(int64_t n, const long long* head, const int32_t* S,
 bool jvp_supports(int method, int problem);
 cudaError_t launch_jvp(int method, int problem, const JvpArgs& a, cudaStream_t s);
 
+// CTAs per SM, lo or hi, for the records whose warps keep their FP64 unit busy (the
+// stiff methods'): c of them take c times one's time for a round of c * wave lanes
+// (wave: a CTA on every SM), so the fewer c * rounds the better; lo on a tie.
+inline int ctas_by_rounds(long long lanes, long long wave, int lo, int hi) {
+  const auto time = [&](int c) { return c * ((lanes + c * wave - 1) / (c * wave)); };
+  return time(hi) < time(lo) ? hi : lo;
+}
+
 struct LaunchCfg {
   int blocks;
   int threads;

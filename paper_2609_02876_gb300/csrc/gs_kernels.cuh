@@ -2080,34 +2080,38 @@ inline cudaError_t fwd_dispatch(const FwdArgs& a_in, cudaStream_t s) {
   }
   if constexpr (stages_possible<M, Pb, R>()) {
     if (a.stages) {
+      const long long wave = (long long)sm_count() * TPB_FWD;
       if constexpr (std::is_same<M, Rodas5PMethod>::value) {
-        // Held to 3 CTAs per SM (168 registers) where those take the ensemble in one
-        // wave and 2 CTAs do not, else with all registers (Robertson: 238, 2 CTAs).
-        // Robertson record, all / 168 registers: 1000 trajectories 2.20 / 2.32 ms;
-        // 40000: 5.26 / 5.01; 56308: 6.42 / 5.08; 65536: 6.52 / 7.66; 2^18: 22.8 / 24.0.
-        const long long wave = (long long)sm_count() * TPB_FWD;
-        if (lanes > 2 * wave && lanes <= 3 * wave)
+        // Held to 168 registers, 3 CTAs per SM, where those take the ensemble in less time, else
+        // with all registers (Robertson: 238, 2 CTAs). Robertson record, all / 168 registers:
+        // 1000 trajectories 2.20 / 2.32 ms; 58000: 6.50 / 4.94; 65536: 6.52 / 7.66; 98000: 9.71
+        // both; 140000: 12.98 / 14.04; 160000: 15.15 / 14.56; 2^18: 22.9 / 24.0; 400000: 34.8 / 33.9.
+        if (ctas_by_rounds(lanes, wave, 2, 3) == 3)
           return persistent_launch(record_kernel_mb<M, Pb, R, true, true, false, 3>, TPB_FWD, smem, lanes, s, &a);
         return persistent_launch(record_kernel_mb<M, Pb, R, true, true, false, 1>, TPB_FWD, smem, lanes, s, &a);
       } else {
-        // Rosenbrock23 (Robertson: 148 registers, 3 CTAs per SM): two waves of 2 CTAs where 3
-        // leave a short second wave. Robertson record of 65536 with 3 / 2: 22.1 / 15.3 ms.
-        const long long wave = (long long)sm_count() * TPB_FWD;
-        const bool two =
-            std::is_same<M, Ros23Method>::value && Pb::D == 3 && lanes > 3 * wave && lanes <= 4 * wave;
-        return persistent_launch(record_kernel<M, Pb, R, true, true>, TPB_FWD, smem, lanes, s, &a, two ? 2 : 1 << 20);
+        // Rosenbrock23 (Robertson: 148 registers, 3 CTAs per SM), 2 / 3 CTAs: 50000 trajectories
+        // 15.1 / 11.6 ms; 66000: 15.3 / 22.1; 78000: 19.7 / 22.4; 82000: 22.4 / 22.5; 140000: 30.3 /
+        // 33.6; 160000: 37.3 / 34.1; 2^18: 53.0 / 56.1; 400000: 82.6 / 79.4. (Held to 128 registers,
+        // 4 CTAs: 66000 17.0, 82000 23.0, 2^18 58.1.)
+        const int most =
+            std::is_same<M, Ros23Method>::value && Pb::D == 3 ? ctas_by_rounds(lanes, wave, 2, 3) : 1 << 20;
+        return persistent_launch(record_kernel<M, Pb, R, true, true>, TPB_FWD, smem, lanes, s, &a, most);
       }
     }
   } else {
     if (a.stages) return cudaErrorInvalidValue;
   }
   int ctas = 1 << 20;
+  const long long wave = (long long)sm_count() * TPB_FWD;
   if constexpr (std::is_same<M, Rodas5PMethod>::value && std::is_same<Pb, NeuralRobertson>::value) {
-    // 3 CTAs per SM fit, and a warp keeps its FP64 unit busy, so a CTA more only costs
-    // where it does not save a wave: records of 65536 trajectories 307 ms with 2 and 438 with
-    // 3, of 56000 220 ms with 3.
-    const long long wave = (long long)sm_count() * TPB_FWD;
-    if (3 * ((lanes + 3 * wave - 1) / (3 * wave)) >= 2 * ((lanes + 2 * wave - 1) / (2 * wave))) ctas = 2;
+    // 3 CTAs per SM fit, and a CTA more only costs where it does not save a round: records of
+    // 65536 trajectories 307 ms with 2 and 438 with 3, of 56000 220 ms with 3.
+    ctas = ctas_by_rounds(lanes, wave, 2, 3);
+  } else if constexpr (std::is_same<M, Ros23Method>::value && std::is_same<Pb, Robertson>::value) {
+    // The compact record without saves (93 registers, 5 CTAs per SM), 4 / 5 CTAs: 90000
+    // trajectories 20.1 / 19.1 ms; 97000: 22.3 / 19.1; 110000: 22.5 / 22.7; 400000: 77.8 / 80.7.
+    if (!a.y_save) ctas = ctas_by_rounds(lanes, wave, 4, 5);
   }
   if (a.y_save) return persistent_launch(record_kernel<M, Pb, R, true, false>, TPB_FWD, smem, lanes, s, &a, ctas);
   return persistent_launch(record_kernel<M, Pb, R, false, false>, TPB_FWD, smem, lanes, s, &a, ctas);

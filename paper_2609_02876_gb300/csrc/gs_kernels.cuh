@@ -1975,8 +1975,9 @@ inline int sm_count() {
 // ensemble needs).
 template <class Kern>
 inline cudaError_t persistent_launch(Kern kern, int tpb, size_t smem, long long n, cudaStream_t s,
-                                     const void* args_ptr, int max_ctas = 1 << 20) {
-  // n: lanes with work; max_ctas: most CTAs per SM
+                                     const void* args_ptr, int max_ctas = 1 << 20,
+                                     unsigned* launched = nullptr) {
+  // n: lanes with work; max_ctas: most CTAs per SM; launched: receives the grid's CTAs
   cudaError_t err = cudaSuccess;
   if (smem > 32 * 1024)  // (static and dynamic together have 48 KB without it)
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1992,6 +1993,7 @@ inline cudaError_t persistent_launch(Kern kern, int tpb, size_t smem, long long 
   }
   if (blocks > need) blocks = need;
   if (blocks < 1) blocks = 1;
+  if (launched) *launched = (unsigned)blocks;
   void* args[] = {const_cast<void*>(args_ptr)};
   return cudaLaunchKernel((const void*)kern, dim3((unsigned)blocks), dim3(tpb), args, smem, s);
 }
@@ -2234,7 +2236,6 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
     using Acc = AccFor<Pb, R>;
     if (a.k != 1) return cudaErrorInvalidValue;
     smem += weight_stage_bytes<Pb>();
-    int bps = 0;
     auto kern = a.y_save_bar ? reverse_k1_entry<M, Pb, R, true>() : reverse_k1_entry<M, Pb, R, false>();
     if constexpr (stages_possible<M, Pb, R>()) {
       if (a.stages) {
@@ -2244,13 +2245,9 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
     } else {
       if (a.stages) return cudaErrorInvalidValue;
     }
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, TPB_REV, smem);
-    cudaError_t e = persistent_launch(kern, TPB_REV, smem, lanes, s, &a);
+    unsigned blocks = 0;  // (every warp of the launched grid writes a partial)
+    cudaError_t e = persistent_launch(kern, TPB_REV, smem, lanes, s, &a, 1 << 20, &blocks);
     if (e != cudaSuccess || !a.wpart || !a.shared_w_bar) return e;
-    long long blocks = (long long)sm_count() * (bps > 0 ? bps : 1);
-    const long long need = (lanes + TPB_REV - 1) / TPB_REV;
-    if (blocks > need) blocks = need;
-    if (blocks < 1) blocks = 1;
     using Part = typename Acc::Part;
     weight_reduce_kernel<Part><<<(Acc::NW + 127) / 128, 128, 0, s>>>(static_cast<const Part*>(a.wpart), Acc::NW,
                                                                       (int)(blocks * (TPB_REV / 32)), a.shared_w_bar);

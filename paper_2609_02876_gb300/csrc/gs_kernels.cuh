@@ -1976,10 +1976,11 @@ inline int sm_count() {
 template <class Kern>
 inline cudaError_t persistent_launch(Kern kern, int tpb, size_t smem, long long n, cudaStream_t s,
                                      const void* args_ptr, int max_ctas = 1 << 20,
-                                     unsigned* launched = nullptr) {
-  // n: lanes with work; max_ctas: most CTAs per SM; launched: receives the grid's CTAs
+                                     unsigned* launched = nullptr, size_t fixed = 16 * 1024) {
+  // n: lanes with work; max_ctas: most CTAs per SM; launched: receives the grid's CTAs;
+  // fixed: the kernel's static shared memory, at most
   cudaError_t err = cudaSuccess;
-  if (smem > 32 * 1024)  // (static and dynamic together have 48 KB without it)
+  if (fixed + smem > 48 * 1024)  // (static and dynamic together have 48 KB without it)
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   const long long need = (n + tpb - 1) / tpb;
@@ -2246,7 +2247,8 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
       if (a.stages) return cudaErrorInvalidValue;
     }
     unsigned blocks = 0;  // (every warp of the launched grid writes a partial)
-    cudaError_t e = persistent_launch(kern, TPB_REV, smem, lanes, s, &a, 1 << 20, &blocks);
+    cudaError_t e =
+        persistent_launch(kern, TPB_REV, smem, lanes, s, &a, 1 << 20, &blocks, 48 * 1024);  // (LvUdeWarp: 42 KB)
     if (e != cudaSuccess || !a.wpart || !a.shared_w_bar) return e;
     using Part = typename Acc::Part;
     weight_reduce_kernel<Part><<<(Acc::NW + 127) / 128, 128, 0, s>>>(static_cast<const Part*>(a.wpart), Acc::NW,

@@ -138,3 +138,16 @@ def test_sharded_weight_gradient_equals_unsharded():
     ref = whole["shared_w_bar"].cpu().numpy().astype(np.float64)
     err = np.abs(summed - ref).max() / np.abs(ref).max()
     assert err < 2e-6, err
+
+
+def test_ude_with_the_most_save_times():
+    """256 saves: the largest dynamic shared memory beside the sweep's 42 KB of static."""
+    wl, w = _setup(300)
+    wl = dict(wl, save_t=np.linspace(wl["t0"], wl["t1"], 257)[1:])
+    rec, _, st = _record(wl, w)
+    assert (st.cpu().numpy() == 0).all()
+    g = _reverse(rec, wl, w)
+    off, h = rec.export_mesh()
+    o = oracle.replay_grad("lv_ude", wl["params"], wl["y0"], wl["t0"], wl["t1"], wl["save_t"], off, h, w=wl["w"])
+    assert_close(g["params_bar"].T, o["params_bar"], "params_bar (a, d)", rtol=TOL)
+    assert_close(g["y0_bar"].T, o["y0_bar"], "y0_bar", rtol=TOL)

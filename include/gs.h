@@ -131,7 +131,10 @@ typedef struct {
                            the device memory allows, and gs_solve_grad for Rodas5P on the
                            neural Robertson up to 12288 trajectories; the reverse sweep then
                            reads the stages instead of recomputing them, with identical
-                           results), else 0 */
+                           results; the neural Robertson's shared_w_bar, an FP64 sum over
+                           the ensemble written out in FP32, may differ in its last bit
+                           where the two layouts run different kernels, from 7169
+                           trajectories on), else 0 */
   int control;          /* GS_CONTROL_FAST or GS_CONTROL_FP64 */
   int record_stages;    /* gs_forward_record only: 1 lets the record also store every step's
                            stage data when gs_solve_grad would (same rule: method, FP64, segment

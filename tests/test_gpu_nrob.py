@@ -137,3 +137,29 @@ def test_nrob_lane_group_and_per_lane_forms(n):
     b = api.solve_grad("nrob", P, Y, wl["t0"], wl["t1"], wl["save_t"], wl["rtol"], wl["atol"], layout="soa",
                        shared_w=SW)
     assert torch.equal(b["params_bar"][:, :m], s["params_bar"]) and torch.equal(b["y0_bar"][:, :m], s["y0_bar"])
+
+
+@pytest.mark.parametrize("n", [7169, 12288])
+def test_nrob_layouts_agree_where_their_kernels_differ(n):
+    """From 7169 to 12288 trajectories stored stages (gs_solve_grad) run 16 lanes
+    per trajectory, compact records (handles, contexts, gs_solve_grad without room
+    for the stages) a lane each: the same operations per trajectory, so the same
+    bits; the weight gradient's FP64 sums run in another order and are written out
+    in FP32, so within an ulp of it."""
+    wl, SW = workload(n)
+    P, Y = dev(wl["params"].T), dev(wl["y0"].T)
+    args = (wl["t0"], wl["t1"], wl["save_t"], wl["rtol"], wl["atol"])
+    info = np.zeros(2, np.int32)
+    s = api.solve_grad("nrob", P, Y, *args, layout="soa", shared_w=SW, record_info=info)
+    assert tuple(info) == (1, 1)
+    ctx = api.Context()
+    c = ctx.solve_grad("nrob", P, Y, *args, layout="soa", shared_w=SW, record_info=info)
+    assert tuple(info) == (1, 0)
+    rec, _, _ = api.forward_record("nrob", P, Y, *args, layout="soa", shared_w=SW, want_saves=False)
+    h = api.reverse(rec, P, Y, layout="soa", shared_w=SW)
+    for r in (c, h):
+        for k in ("loss", "params_bar", "y0_bar"):
+            assert torch.equal(s[k], r[k]), k
+        d = (s["shared_w_bar"].double() - r["shared_w_bar"].double()).abs()
+        assert (d <= 2.0 ** -23 * s["shared_w_bar"].double().abs().max()).all()
+    ctx.close()

@@ -8,6 +8,7 @@ import torch
 
 from paper_2609_02876_gb300 import api, build
 from paper_2609_02876_gb300 import workloads as W
+from tests.test_gpu_queueing import args, long_lorenz
 from tests.test_gpu_tsit5 import dev
 
 pytestmark = pytest.mark.gpu
@@ -80,3 +81,56 @@ def test_options_and_failed_trajectories(kw):
     p[200] = 0.0
     st = both("lorenz", p, y, wl["t0"], wl["t1"], wl["save_t"], wl["rtol"], wl["atol"], **kw)
     assert (st[[3, 64, 95]] == 3).all()
+
+
+@pytest.mark.parametrize("n", [1, 700, 20011])
+@pytest.mark.parametrize("in_place", [False, True])
+def test_overflowing_packed_arena_reruns_record_and_sweep(n, in_place):
+    wl = long_lorenz(n)
+    build.build()
+    P, Y = dev(wl["params"].T), dev(wl["y0"].T)
+    rec, _, _ = api.forward_record("lorenz", P, Y, *args(wl), layout="soa", want_saves=False, ckpt_k=1,
+                                   precision="fp32_mixed")
+    ref = api.reverse(rec, P, Y, layout="soa")
+    p, y = P.clone(), Y.clone()
+    out = {"loss": torch.empty(n, dtype=torch.float64, device="cuda"),
+           "params_bar": p if in_place else torch.empty_like(P), "y0_bar": y if in_place else torch.empty_like(Y),
+           "status": torch.empty(n, dtype=torch.int32, device="cuda")}
+    ctx = api.Context()  # a workspace of its own, so its first arena is the expected size
+    g = ctx.solve_grad("lorenz", p, y, *args(wl), layout="soa", out=out, precision="fp32_mixed")
+    assert (g["status"] == 0).all()
+    for k in ("loss", "params_bar", "y0_bar"):
+        assert torch.equal(g[k], ref[k]), k
+    ctx.close()
+
+
+def test_more_segments_than_a_packed_index_holds():
+    """2.0e9 accepted steps where 2.1e8 were expected: past a packed segment's
+    31-bit index, so the rerun is over general segments (about 110 GB)."""
+    build.build()
+    n = 1 << 21
+    wl = W.make("vdp", n)
+    P, Y = dev(wl["params"].T), dev(wl["y0"].T)
+
+    def grad(ctx, lo, hi, t1, **kw):
+        saves = np.linspace(0.0, t1, 6)[1:]
+        return ctx.solve_grad("vdp", P[:, lo:hi].contiguous(), Y[:, lo:hi].contiguous(), 0.0, t1, saves, wl["rtol"],
+                              wl["atol"], layout="soa", precision="fp32_mixed", **kw)
+
+    ctx = api.Context()
+    m = 1 << 17  # a packed sample gives the steps per unit of time
+    s = grad(ctx, 0, m, 100.0, step_counts=True)["step_counts"][0].double().mean().item()
+    t1 = 100.0 * 2.0e9 / (s * n)
+    part = grad(ctx, n - m, n, t1, step_counts=True)
+    total = part["step_counts"][0].double().mean().item() * n
+    assert 1.93e9 < total < 2.1e9
+    ctx.close()
+    torch.cuda.empty_cache()
+    ctx = api.Context()
+    g = grad(ctx, 0, n, t1)
+    assert (g["status"] == 0).all()
+    for k in ("loss", "params_bar", "y0_bar", "status"):
+        assert torch.equal(g[k][..., n - m:], part[k]), k
+    used = torch.cuda.mem_get_info()[0]
+    ctx.close()
+    assert torch.cuda.mem_get_info()[0] - used > (90 << 30)  # the arena was the general one

@@ -2227,6 +2227,15 @@ inline cudaError_t order_pass(RevArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Sweeps of records with k > 1.
+template <class M, class Pb, class R>
+inline cudaError_t rev_many_dispatch(const RevArgs& a, cudaStream_t s) {
+  if (a.k == 1 || a.stages) return cudaErrorInvalidValue;
+  const size_t smem = (size_t)((a.n_save + 1) & ~1) * sizeof(double);
+  if (a.y_save_bar) return persistent_launch(reverse_kernel<M, Pb, R, true>, TPB_REV, smem, a.n, s, &a);
+  return persistent_launch(reverse_kernel<M, Pb, R, false>, TPB_REV, smem, a.n, s, &a);
+}
+
 template <class M, class Pb, class R, bool SOFT = false>
 inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
   RevArgs a = a_in;
@@ -2240,8 +2249,9 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
     auto kern = a.y_save_bar ? reverse_k1_entry<M, Pb, R, true>() : reverse_k1_entry<M, Pb, R, false>();
     if constexpr (stages_possible<M, Pb, R>()) {
       if (a.stages) {
-        if (a.segw != stage_segw<M, Pb::D>()) return cudaErrorInvalidValue;
-        kern = a.y_save_bar ? reverse_k1_entry<M, Pb, R, true, true>() : reverse_k1_entry<M, Pb, R, false, true>();
+        // (gs_solve_grad's own records: the built-in loss)
+        if (a.segw != stage_segw<M, Pb::D>() || a.y_save_bar) return cudaErrorInvalidValue;
+        kern = reverse_k1_entry<M, Pb, R, false, true>();
       }
     } else {
       if (a.stages) return cudaErrorInvalidValue;
@@ -2300,12 +2310,10 @@ inline cudaError_t rev_dispatch(const RevArgs& a_in, cudaStream_t s) {
     if (a.y_save_bar) return persistent_launch(reverse_k1_entry<M, Pb, R, true>(), TPB_REV, smem, lanes, s, &a, ctas);
     return persistent_launch(reverse_k1_entry<M, Pb, R, false>(), TPB_REV, smem, lanes, s, &a, ctas);
   }
-  if constexpr (GroupOf<Pb>::value > 1) {
+  if constexpr (GroupOf<Pb>::value > 1)
     return cudaErrorInvalidValue;  // (lane groups sweep k = 1 records)
-  } else {
-    if (a.y_save_bar) return persistent_launch(reverse_kernel<M, Pb, R, true>, TPB_REV, smem, lanes, s, &a);
-    return persistent_launch(reverse_kernel<M, Pb, R, false>, TPB_REV, smem, lanes, s, &a);
-  }
+  else
+    return rev_many_dispatch<M, Pb, R>(a, s);
   }
   }
 }

@@ -46,9 +46,7 @@ cudaError_t launch_tsit5_forward(int problem, int precision, const FwdArgs& a, c
   switch (problem * 2 + precision) {
     case 0: return fwd_dispatch<Tsit5Method, Lorenz, double>(a, s);
     case 1: return fwd_dispatch<Tsit5Method, Lorenz, float>(a, s);
-    case 2: return fwd_dispatch<Tsit5Method, VanDerPol, double>(a, s);
     case 3: return fwd_dispatch<Tsit5Method, VanDerPol, float>(a, s);
-    case 8: return fwd_dispatch<Tsit5Method, Linear2, double>(a, s);
     case 9: return fwd_dispatch<Tsit5Method, Linear2, float>(a, s);
     case 11: return fwd_dispatch<Tsit5Method, LvUde, float>(a, s);
   }
@@ -61,9 +59,9 @@ cudaError_t launch_tsit5_reverse(int problem, int precision, const RevArgs& a, c
   switch (problem * 2 + precision) {
     case 0: return rev_dispatch<Tsit5Method, Lorenz, double>(a, s);
     case 1: return rev_dispatch<Tsit5Method, Lorenz, float>(a, s);
-    case 2: return rev_dispatch<Tsit5Method, VanDerPol, double>(a, s);
+    case 2: return rev_many_dispatch<Tsit5Method, VanDerPol, double>(a, s);  // (k = 1: soft_launch)
     case 3: return rev_dispatch<Tsit5Method, VanDerPol, float>(a, s);
-    case 8: return rev_dispatch<Tsit5Method, Linear2, double>(a, s);
+    case 8: return rev_many_dispatch<Tsit5Method, Linear2, double>(a, s);
     case 9: return rev_dispatch<Tsit5Method, Linear2, float>(a, s);
 #if GS_UDE_CTA
     case 11: return rev_dispatch<Tsit5Method, LvUdeCta, float>(a, s);  // CTA-collective network (tcgen05)

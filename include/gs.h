@@ -370,7 +370,7 @@ gs_status gs_record_stats(const gs_record* rec, int64_t* n, int64_t* accepted, i
  * Synchronous. Meant for tests and inspection. */
 gs_status gs_record_export_mesh(const gs_record* rec, int64_t* offsets, double* h);
 
-/* Releases a record (NULL is accepted) after the device's queued work. The device
+/* Releases a record (NULL is accepted); work queued on it still completes. The device
  * buffers of up to two freed records, of at most 128 MB each, stay with the library
  * for a later gs_forward_record of the same problem, options, n, n_save and rtol; they
  * are given back when newer ones take their place or an allocation of the library

@@ -151,6 +151,16 @@ struct gs_record {
   mutable long long* fwd_base = nullptr;
   mutable long long* fwd_seg = nullptr;
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // kernel timing (optional)
+  // A handle's last use on each stream (the streams' ids, which are never used again), for
+  // the pool; once not all of them are known (a captured use, too many streams) it does not
+  // enter the pool.
+  struct Use {
+    unsigned long long stream;
+    cudaEvent_t done;
+  };
+  mutable std::mutex use_mu;
+  mutable std::vector<Use> uses;
+  mutable bool uses_known = true;
 };
 
 // A solve context: its own reusable record workspace, so that calls on
@@ -253,6 +263,7 @@ void destroy(gs_record* r) {
   if (!r) return;
   for (int i = 0; i < 4; ++i)
     if (r->ev[i]) cudaEventDestroy(r->ev[i]);
+  for (const gs_record::Use& u : r->uses) cudaEventDestroy(u.done);
   free_arrays(r);
   cudaFree(r->arena);
   cudaFree(r->fwd_base);
@@ -272,26 +283,63 @@ void destroy(gs_record* r) {
 // the library holds beside the caller's allocator, 256 MB in all; with 10 saves a
 // Lorenz record stays below them up to about 12300 trajectories, with 50 saves a Van
 // der Pol record up to about 7100. At most POOL_RECORDS of them; the oldest is
-// released for a newer one, and all of them when an allocation fails. A record
-// enters the pool after the device has finished all work, as cudaFree would have
-// waited for, so any stream may use it next.
+// released for a newer one, and all of them when an allocation fails. The call that
+// takes a record waits for the uses it was freed with (an event per stream): a free
+// itself waits for nothing, and unlike a wait for the device neither breaks a capture
+// that another stream has under way.
 constexpr size_t POOL_RECORD_BYTES = size_t(128) << 20;
 constexpr size_t POOL_RECORDS = 2;
+constexpr size_t POOL_STREAMS = 8;
 std::mutex g_pool_mu;
 std::vector<gs_record*> g_pool;  // oldest first
+
+// Notes that work on record r has been queued on stream s.
+void note_use(const gs_record* r, cudaStream_t s) {
+  std::lock_guard<std::mutex> lock(r->use_mu);
+  if (!r->uses_known) return;
+  r->uses_known = false;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
+  unsigned long long id = 0;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return;
+  if (cudaStreamGetId(s, &id) != cudaSuccess) return;
+  cudaEvent_t done = nullptr;
+  for (const gs_record::Use& u : r->uses)
+    if (u.stream == id) done = u.done;
+  if (!done) {
+    if (r->uses.size() >= POOL_STREAMS) return;
+    if (cudaEventCreateWithFlags(&done, cudaEventDisableTiming) != cudaSuccess) return;
+    try {
+      r->uses.push_back({id, done});
+    } catch (...) {
+      cudaEventDestroy(done);
+      return;
+    }
+  }
+  r->uses_known = cudaEventRecord(done, s) == cudaSuccess;
+}
 
 gs_record* pool_take(const RecordKey& key) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
-  std::lock_guard<std::mutex> lock(g_pool_mu);
-  for (size_t i = 0; i < g_pool.size(); ++i) {
-    gs_record* r = g_pool[i];
-    if (r->device == dev && r->key == key) {
-      g_pool.erase(g_pool.begin() + i);
-      return r;
-    }
+  gs_record* r = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    for (size_t i = 0; i < g_pool.size() && !r; ++i)
+      if (g_pool[i]->device == dev && g_pool[i]->key == key) {
+        r = g_pool[i];
+        g_pool.erase(g_pool.begin() + i);
+      }
   }
-  return nullptr;
+  if (!r) return nullptr;
+  for (const gs_record::Use& u : r->uses)
+    if (cudaEventSynchronize(u.done) != cudaSuccess) {
+      destroy(r);
+      return nullptr;
+    }
+  cudaFree(r->fwd_base);
+  cudaFree(r->fwd_seg);
+  r->fwd_base = r->fwd_seg = nullptr;
+  return r;
 }
 
 bool pool_put(gs_record* r) {  // false: the caller releases it
@@ -299,11 +347,7 @@ bool pool_put(gs_record* r) {  // false: the caller releases it
   const size_t partials = r->wpart ? (size_t)ude_max_warps() * WPART_BYTES_PER_WARP : 0;
   if (record_bytes(r) + partials > POOL_RECORD_BYTES) return false;
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev != r->device) return false;
-  if (cudaDeviceSynchronize() != cudaSuccess) return false;
-  cudaFree(r->fwd_base);
-  cudaFree(r->fwd_seg);
-  r->fwd_base = r->fwd_seg = nullptr;
+  if (!r->uses_known || cudaGetDevice(&dev) != cudaSuccess || dev != r->device) return false;
   gs_record* old = nullptr;
   try {
     std::lock_guard<std::mutex> lock(g_pool_mu);
@@ -1070,8 +1114,10 @@ gs_status gs_reverse(const gs_record* rec, const double* params, const double* y
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev != rec->device) return GS_ERR_INVALID_ARG;
-  return launch_reverse(rec, params, shared_w, y_save_bar, loss_out, params_bar, y0_bar, shared_w_bar, rec->status,
-                        false, (cudaStream_t)stream);
+  const gs_status st = launch_reverse(rec, params, shared_w, y_save_bar, loss_out, params_bar, y0_bar, shared_w_bar,
+                                      rec->status, false, (cudaStream_t)stream);
+  note_use(rec, (cudaStream_t)stream);
+  return st;
 }
 
 gs_status gs_replay_jvp(const gs_record* rec, const double* params, const double* y0, int n_dir,
@@ -1087,7 +1133,9 @@ gs_status gs_replay_jvp(const gs_record* rec, const double* params, const double
   a.y0_dot = y0_dot;
   a.loss_dot = loss_dot;
   a.y_save_dot = y_save_dot;
-  return launch_jvp_range(rec, a, 0, n_dir, loss_out, (cudaStream_t)stream);
+  const gs_status sl = launch_jvp_range(rec, a, 0, n_dir, loss_out, (cudaStream_t)stream);
+  note_use(rec, (cudaStream_t)stream);
+  return sl;
 }
 
 gs_status gs_forward_grad(const gs_record* rec, const double* params, const double* y0, double* loss_out,
@@ -1103,7 +1151,9 @@ gs_status gs_forward_grad(const gs_record* rec, const double* params, const doub
   a.grad_y = y0_bar;
   const int g0 = params_bar ? 0 : rec->P;
   const int g1 = y0_bar ? rec->P + rec->d : rec->P;
-  return launch_jvp_range(rec, a, g0, g1, loss_out, (cudaStream_t)stream);
+  const gs_status sl = launch_jvp_range(rec, a, g0, g1, loss_out, (cudaStream_t)stream);
+  note_use(rec, (cudaStream_t)stream);
+  return sl;
 }
 
 gs_status gs_record_refresh(gs_record* rec, const double* params, const double* y0, const float* shared_w,
@@ -1139,6 +1189,7 @@ gs_status gs_record_refresh(gs_record* rec, const double* params, const double* 
       : (rec->method == GS_METHOD_VERNER7)
           ? launch_vern7_refresh(rec->problem, rec->precision, a, rec->arena, rec->y_final, y0, s)
           : launch_tsit5_refresh(rec->problem, rec->precision, a, rec->arena, rec->y_final, y0, s);
+  note_use(rec, s);
   return e == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 

@@ -88,3 +88,57 @@ def test_records_from_the_pool_equal_fresh_ones():
     r4, _, _ = api.forward_record("lorenz", P[:, :33].contiguous(), Y[:, :33].contiguous(), *args(wl), **kw)
     assert torch.equal(api.reverse(r4, P[:, :33].contiguous(), Y[:, :33].contiguous(), layout="soa")["params_bar"],
                        g0["params_bar"][:, :33])
+
+
+def test_freeing_a_record_leaves_a_capture_alone():
+    """A record may be freed (by the collector, say) while a stream captures in
+    the relaxed mode; a sweep may be captured, and its record freed after the graph."""
+    wl = W.make("lorenz", 2003)
+    P, Y = dev(wl["params"].T), dev(wl["y0"].T)
+    rec, _, _ = api.forward_record("lorenz", P, Y, *args(wl), layout="soa")
+    ref = api.reverse(rec, P, Y, layout="soa")
+    swept, _, _ = api.forward_record("lorenz", P, Y, *args(wl), layout="soa")
+    torch.cuda.synchronize()
+    graph, x = torch.cuda.CUDAGraph(), torch.zeros(4, device="cuda")
+    with torch.cuda.graph(graph, capture_error_mode="relaxed"):
+        x.add_(1)
+        rec.free()
+        g = api.reverse(swept, P, Y, layout="soa")
+        x.add_(1)
+    other, _, _ = api.forward_record("lorenz", 1.01 * P, Y, *args(wl), layout="soa")  # through the pool
+    graph.replay()
+    torch.cuda.synchronize()
+    assert (x == 2).all()
+    for k in ("loss", "params_bar", "y0_bar"):
+        assert torch.equal(g[k], ref[k]), k
+    del graph
+    swept.free()
+    other.free()
+
+
+@pytest.mark.parametrize("streams", [1, 3, 11])
+def test_a_record_from_the_pool_waits_for_its_sweeps(streams):
+    """A record freed with long sweeps queued on several streams, and its buffers
+    taken by a record of other inputs on another stream: the sweeps' results stand."""
+    wl = W.make("lorenz", 4001)
+    P, Y = dev(wl["params"].T), dev(wl["y0"].T)
+    kw = dict(layout="soa", record_stages=True)
+    rec, _, _ = api.forward_record("lorenz", P, Y, *args(wl), **kw)
+    ref = api.reverse(rec, P, Y, layout="soa")
+    torch.cuda.synchronize()
+    ss = [torch.cuda.Stream() for _ in range(streams)]
+    out = []
+    for s in ss:  # one stream's sweeps after the other's (a sweep's tickets are the record's own)
+        s.wait_stream(torch.cuda.current_stream() if not out else prev)
+        with torch.cuda.stream(s):
+            out += [api.reverse(rec, P, Y, layout="soa") for _ in range(24 // streams)]
+        prev = s
+    rec.free()
+    taker = torch.cuda.Stream()
+    with torch.cuda.stream(taker):
+        r2, _, _ = api.forward_record("lorenz", 1.5 * P, 0.5 * Y, *args(wl), **kw)
+    torch.cuda.synchronize()
+    for g in out:
+        for k in ("loss", "params_bar", "y0_bar"):
+            assert torch.equal(g[k], ref[k]), k
+    r2.free()

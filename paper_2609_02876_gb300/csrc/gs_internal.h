@@ -13,7 +13,8 @@ constexpr int KMAX_HOST = 32;  // largest checkpoint interval accepted by the AB
 // per lane in shared memory (128 lanes).
 constexpr int MAX_STAGE_SEGW = 72;
 // The neural Robertson: the largest ensembles in the lane-group form (gs_nrob.cu)
-// without and with stored stages, which it alone has, and the doubles that a
+// without and with stored stages, which it alone has (where its time, proportional to
+// the ensemble, met that of a lane per trajectory on 152 SMs), and the doubles that a
 // step's stage data takes there.
 constexpr int64_t NR_GROUP_MAX = 7168, NR_GROUP_STAGES_MAX = 12288;
 constexpr int NRG_STAGE_DOUBLES = 330;

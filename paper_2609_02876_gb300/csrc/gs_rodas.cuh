@@ -196,7 +196,7 @@ struct ContractOf<Pb, std::void_t<typename Pb::Contract>> {
 };
 
 // ---------------------------------------------------------------------------
-// The same for a matrix whose structural zeros are known (HIRES: 24 of W's 64
+// The same for a matrix whose structural zeros are known (HIRES: 25 of W's 64
 // entries). With partial pivoting the row exchanged at column k is one of those
 // with an entry in it, so the entries that the factors can hold are bounded at
 // compile time: u[k][j] for row k of U, l[i][k] for the multipliers of column k

@@ -22,22 +22,22 @@ bool tsit5_supports(int problem, int precision) {
 
 // Other FP64 launches in soft arithmetic (SoftD, multiplications on the integer
 // pipes): every ensemble of the two-dimensional problems, and ensembles of more
-// than one warp per FP64 unit (19456 trajectories) of the three-dimensional
+// than one warp per FP64 unit (four per SM: 19456 trajectories) of the three-dimensional
 // ones. Gradient of n trajectories, record + reverse, hardware against soft:
 // Lorenz 10007: 0.99 / 0.99 ms; 26000: 1.56 / 1.33; 60000: 3.07 / 2.37; 2^22:
 // 151.7 / 120.4; Van der Pol 700: 2.26 / 2.12 ms; 26000: 3.44 / 2.87; 65521: 6.83
 // / 5.01; 2^20: 73.1 / 53.5.
 bool soft_launch(int problem, int precision, int64_t n) {
-  return precision == 0 && (problem == 1 || problem == 4 || n > 608 * 32);
+  return precision == 0 && (problem == 1 || problem == 4 || n > 4ll * sm_count() * 32);
 }
 
 // FP64 launches with a lane per state component (gs_group.cuh): Lorenz and Van
-// der Pol up to 9728 trajectories (Lorenz: two group warps per FP64 unit; Van der
-// Pol: one). Gradient, record + reverse, per-lane against groups: Lorenz 1024:
+// der Pol up to 16 trajectories per FP64 unit, 9728 (Lorenz: two group warps per unit;
+// Van der Pol: one). Gradient, record + reverse, per-lane against groups: Lorenz 1024:
 // 0.96 / 0.64 ms; 9728: 0.99 / 0.85; 10007: 0.99 / 1.15 (some units hold three);
 // Van der Pol 700: 2.12 / 1.95; 9728: 2.24 / 2.04; 14000: 2.26 / 2.64.
 bool group_launch(int problem, int precision, int64_t n) {
-  return precision == 0 && (problem == 0 || problem == 1) && n <= 9728;
+  return precision == 0 && (problem == 0 || problem == 1) && n <= 4ll * sm_count() * 16;
 }
 
 cudaError_t launch_tsit5_forward(int problem, int precision, const FwdArgs& a, cudaStream_t s) {

@@ -167,7 +167,8 @@ gs_status gs_problem_info(int problem_id, int* d, int* P, int* stiff, int* n_sha
  * shared_w: the network weights of GS_LV_UDE (354 floats) or
  * GS_NEURAL_ROBERTSON (353 floats), device, else NULL.
  * traj_status [n] is required. Synchronises `stream`. The record stays valid
- * until gs_record_free and may be replayed any number of times.
+ * until gs_record_free and may be replayed any number of times, on any streams, one
+ * sweep after another (sweeps of one record share its counters and must not overlap).
  */
 gs_status gs_forward_record(int problem_id, int64_t n, const double* params, const double* y0,
                             const float* shared_w, double t0, double t1, const double* save_t, int n_save,

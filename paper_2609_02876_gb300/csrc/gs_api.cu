@@ -744,7 +744,7 @@ gs_status launch_reverse(const gs_record* r, const double* params, const float* 
   a.S = r->S;
   a.y_final = r->y_final;
   a.wpart = r->wpart;
-  a.order_buf = r->order_cap >= r->n ? r->order : nullptr;  // (workspaces: a handle may be swept on several streams)
+  a.order_buf = r->order_cap >= r->n ? r->order : nullptr;  // (workspaces)
   a.work = &r->ctr->work_rev;
   a.k = r->k;
   a.segw = r->segw;
